@@ -28,6 +28,8 @@ struct LjConsts {
   float rho_f, rho_re_f, m_g_f, m_half_f;
   float rho_lo;         // rho - rho_f: rho as a double-float (rho_f, rho_lo)
   float eps_f;          // eps: energy factor of a half-pair sum
+  float re_f;           // re
+  float m_slope2_f;     // (rho / re) log2 e: slope of the exponent to base 2
 };
 
 inline LjConsts make_consts(double eps, double sigma, int pot = 0, double rho = 0.0) {
@@ -58,6 +60,8 @@ inline LjConsts make_consts(double eps, double sigma, int pot = 0, double rho = 
   k.m_half_f = (float)k.m_half;
   k.rho_lo = (float)(rho - (double)k.rho_f);
   k.eps_f = (float)eps;
+  k.re_f = (float)sigma;
+  k.m_slope2_f = (float)(k.rho_re * 1.4426950408889634074);
   return k;
 }
 

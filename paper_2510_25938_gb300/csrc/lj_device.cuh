@@ -309,6 +309,45 @@ __device__ __forceinline__ float rcp_approx(float x) {
   return r;
 }
 
+__device__ __forceinline__ float rsqrt_approx(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float ex2_approx(float x) {
+  float r;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
+// 1 / a in FP64: the hardware's estimate r (PTX rcp.approx.ftz.f64, ~2^-20
+// relative) and one third-order Householder step, r (1 + e + e^2) with
+// e = 1 - a r formed by one FMA: the truncation error e^3 is below 2^-58, so the
+// result is within an ulp of 1 / a.  Three FP64 instructions, against about
+// nine of the correctly rounded reciprocal, and none on the FP64 pipe for the
+// ends of the range: an estimate of 0 or infinity (a = 0, infinite or so small
+// that its inverse overflows) is returned as it is, chosen by its exponent
+// bits on the integer pipe.
+__device__ __forceinline__ bool f64_end(double r) {   // 0, subnormal, infinite or NaN
+  const int ex = __double2hiint(r) & 0x7ff00000;
+  return ex == 0 || ex == 0x7ff00000;
+}
+__device__ __forceinline__ double rcp_f64(double a, double one = 1.0) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
+  const double e = fma(-a, r, one);
+  const double y = fma(r, fma(e, e, e), r);
+  return f64_end(r) ? r : y;
+}
+// 1 / sqrt(a) in FP64, likewise: with e = 1 - a r^2, r (1 + e/2 + 3 e^2 / 8)
+__device__ __forceinline__ double rsqrt_f64(double a) {
+  double r;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
+  const double e = fma(-(a * r), r, 1.0);
+  const double y = fma(r * e, fma(0.375, e, 0.5), r);
+  return f64_end(r) ? r : y;
+}
+
 struct alignas(16) PosF { float x, y, z, w; };
 struct alignas(16) PosD { double x, y, z, w; };
 
