@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(256, 2) eval_ring_f32_kernel(ljh::EvalArgs a, 
       }
       NG = (n + G - 1) / G;
       H = NG >> 1;
-      P = NG > 0 ? max(1, min(B / NG, (H + S - 1) / S)) : 1;
+      P = NG > 0 ? max(1, min(B / NG, (H + S - 1) / S + 1)) : 1;
       place();
     }
     const bool live = lc < pl.C && c0 + lc < a.n_cand;
@@ -189,7 +189,7 @@ __global__ void __launch_bounds__(256, POT == LJ_POT_LJ ? 2 : 1) eval_ring_f64_k
       }
       NG = (n + G - 1) / G;
       H = NG >> 1;
-      P = NG > 0 ? max(1, min(B / NG, (H + S - 1) / S)) : 1;
+      P = NG > 0 ? max(1, min(B / NG, (H + S - 1) / S + 1)) : 1;
       place();
     }
     const bool live = lc < pl.C && c0 + lc < a.n_cand;
@@ -244,50 +244,68 @@ __global__ void __launch_bounds__(256, POT == LJ_POT_LJ ? 2 : 1) eval_ring_f64_k
         }
       }
     }
-    auto put = [&](PosDG<G>& w) {
+    if (P == 1 && S == 1) {
+      if (live && gout) {
+        IO* go = gout + 3 * a0;
+#pragma unroll
+        for (int j = 0; j < G; ++j) {
+          const int i = G * g + j;
+          if (i < n) {
+            go[3 * i] = (IO)(gs * f.x[j]);
+            go[3 * i + 1] = (IO)(gs * f.y[j]);
+            go[3 * i + 2] = (IO)(gs * f.z[j]);
+          }
+        }
+      }
+      if (tid < 32)
+        sum_energies(es, pl.C, NG, [&](int c, dd s) {
+          if (c0 + c < a.n_cand) a.energy[c0 + c] = total(s) * ef;
+        });
+      continue;
+    }
+    // parts in the order of p, then CTAs in the order of s, one coordinate a
+    // thread (C = 1 here); the energies by the last warp meanwhile
+    if (live) {
+      PosDG<G>& w = own[slot + g];
 #pragma unroll
       for (int j = 0; j < G; ++j) { w.x[j] = f.x[j]; w.y[j] = f.y[j]; w.z[j] = f.z[j]; }
-    };
-    auto add = [&](const PosDG<G>& r) {
-#pragma unroll
-      for (int j = 0; j < G; ++j) { f.x[j] += r.x[j]; f.y[j] += r.y[j]; f.z[j] += r.z[j]; }
-    };
-    if (P > 1) {
-      if (live && p > 0) put(own[slot + g]);
-      __syncthreads();
-      if (live && p == 0)
-        for (int pp = 1; pp < P; ++pp) add(own[slot + pp * NG + g]);
     }
-    if (tid < 32)
-      sum_energies(es, pl.C, NG * P, [&](int c, dd s) {
-        if (S > 1) ecl[c] = s;
-        else if (c0 + c < a.n_cand) a.energy[c0 + c] = total(s) * ef;
+    __syncthreads();
+    constexpr int D = sizeof(PosDG<G>) / sizeof(double);   // doubles a slot, 3 G used
+    double* od = reinterpret_cast<double*>(own);
+    const long long first = a.uniform_n > 0 ? c0 * n : a0;   // of any thread, live or not
+    auto out = [&](int o, double v) {        // coordinate o: group, axis, atom of the group
+      const int i = G * (o / (3 * G)) + o % G, ax = o % (3 * G) / G;
+      if (gout && i < n) gout[3 * (first + i) + ax] = (IO)(gs * v);
+    };
+    for (int o = tid; o < 3 * G * NG; o += B) {
+      double* q0 = od + (o / (3 * G)) * D + o % (3 * G);
+      double v = *q0;
+      for (int pp = 1; pp < P; ++pp) v += q0[(size_t)pp * NG * D];
+      if (S == 1) out(o, v);
+      else *q0 = v;
+    }
+    if (tid >= B - 32)
+      sum_energies(es, 1, NG * P, [&](int, dd s) {
+        if (S > 1) ecl[0] = s;
+        else a.energy[c0] = total(s) * ef;
       });
     if (S > 1) {
       cg::cluster_group cl = cg::this_cluster();
-      if (live && p == 0) put(own[slot + g]);
       cl.sync();
-      group_zero(f);
-      if (live && p == 0 && g % S == srank)
-        for (int s = 0; s < S; ++s) add(*cl.map_shared_rank(&own[slot + g], s));
-      if (srank == 0 && tid < pl.C && c0 + tid < a.n_cand) {
-        dd s = ecl[tid];
-        for (int r = 1; r < S; ++r) acc_pair(s, *cl.map_shared_rank(&ecl[tid], r));
-        a.energy[c0 + tid] = total(s) * ef;
+      for (int o = tid; o < 3 * G * NG; o += B) {
+        if (o / (3 * G) % S != srank) continue;
+        double* q0 = od + (o / (3 * G)) * D + o % (3 * G);
+        double v = 0.0;
+        for (int s = 0; s < S; ++s) v += *cl.map_shared_rank(q0, s);
+        out(o, v);
+      }
+      if (srank == 0 && tid == 0) {
+        dd s = ecl[0];
+        for (int r = 1; r < S; ++r) acc_pair(s, *cl.map_shared_rank(&ecl[0], r));
+        a.energy[c0] = total(s) * ef;
       }
       cl.sync();
-    }
-    if (live && gout && p == 0 && (S == 1 || g % S == srank)) {
-      IO* go = gout + 3 * a0;
-#pragma unroll
-      for (int j = 0; j < G; ++j) {
-        const int i = G * g + j;
-        if (i < n) {
-          go[3 * i] = (IO)(gs * f.x[j]);
-          go[3 * i + 1] = (IO)(gs * f.y[j]);
-          go[3 * i + 2] = (IO)(gs * f.z[j]);
-        }
-      }
     }
   }
 }
@@ -358,7 +376,7 @@ RingLaunch ring_plan(const ljh::EvalArgs& a, int sms) {
   } else if (a.uniform_n > 0) {
     // few candidates: more parts until the threads fill the GPU
     const long long more = want / (a.n_cand * NG);
-    pl.P = (int)std::max(1LL, std::min<long long>(std::min(more, (long long)NG / 2), kRingMaxB / NG));
+    pl.P = (int)std::max(1LL, std::min<long long>(std::min(more, (long long)NG / 2 + 1), kRingMaxB / NG));
     r.B = (NG * pl.P + 31) / 32 * 32;
   } else {
     // uneven: one candidate a CTA, its parts set by the kernel from its own size

@@ -68,10 +68,13 @@ static_assert(sizeof(PosDG<2>) == 48 && sizeof(PosDG<4>) == 96 && sizeof(SlotF<4
 // the first warp in a fixed order: L lanes a candidate, strided, then a tree
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void acc_pair(ff& s, ff v) { df_acc(s, v); }
+// TwoSum with the operands ordered by magnitude on the integer pipe: three
+// FP64 additions (Dekker's FastTwoSum) instead of six
 __device__ __forceinline__ void acc_pair(dd& s, dd v) {
-  const dd t = dd_two_sum(s.hi, v.hi);
-  s.hi = t.hi;
-  s.lo = __dadd_rn(s.lo, __dadd_rn(t.lo, v.lo));
+  const bool sw = (__double2hiint(s.hi) & 0x7fffffff) < (__double2hiint(v.hi) & 0x7fffffff);
+  const double a = sw ? v.hi : s.hi, b = sw ? s.hi : v.hi;
+  s.hi = __dadd_rn(a, b);
+  s.lo = __dadd_rn(s.lo, __dadd_rn(__dsub_rn(b, __dsub_rn(s.hi, a)), v.lo));
 }
 __device__ __forceinline__ double total(ff s) { return (double)s.hi + (double)s.lo; }
 __device__ __forceinline__ double total(dd s) { return __dadd_rn(s.hi, s.lo); }
@@ -79,7 +82,7 @@ __device__ __forceinline__ double total(dd s) { return __dadd_rn(s.hi, s.lo); }
 template <typename E, typename F>
 __device__ __forceinline__ void sum_energies(const E* es, int C, int cnt, F&& store) {
   int L = 32;
-  while (L > 1 && L * C > 32) L >>= 1;
+  while (L > 1 && (L * C > 32 || L >= 2 * cnt)) L >>= 1;
   const int lane = threadIdx.x & 31, sub = lane & (L - 1), per = 32 / L;
   for (int c0 = 0; c0 < C; c0 += per) {
     const int c = c0 + lane / L;
