@@ -35,7 +35,8 @@ __device__ __forceinline__ MinParams to_dev(const ljh::MinParamsH& h) {
   p.gtol = h.gtol; p.c1 = h.c1; p.c2 = h.c2; p.alpha_max = h.alpha_max;
   p.switch_gtol = h.switch_gtol; p.deadline = h.deadline; p.k = h.k;
   p.f32_resolution = h.f32_resolution; p.df_resolution = h.df_resolution;
-  p.tiled = 0;
+  p.layout = 0;
+  p.ring_ks = 1;
   return p;
 }
 
@@ -85,9 +86,10 @@ __global__ void __launch_bounds__(T, T <= 64 ? 3 : 0) bh_cluster_kernel(ljh::BhA
   carve_team<T>(sp, n, true, a.hist_on_chip ? a.hist_slot_bytes : 0, pos, hbuf, hist, tm.red,
                 word);
   MinParams p = to_dev(a.p);
-  // hbuf: pair buffer up to 64 atoms, tile accumulators above 256; with
+  // hbuf: pairs up to 64 atoms, ring chunks up to 256, tile accumulators above; with
   // one-sided rows chosen above 256 atoms it holds no pairs and is withdrawn
-  p.tiled = n > kTileMinN && !a.p.df_one_sided;
+  p.layout = pair_layout(n);
+  p.ring_ks = ring_shifts(n);
   if (n > kTileMinN && a.p.df_one_sided) hbuf = nullptr;
   if (!a.hist_on_chip)
     hist = static_cast<unsigned char*>(a.hist) + ((size_t)w * K + k) * a.hist_slot_bytes;
@@ -247,7 +249,7 @@ cudaError_t plan_one(int n_atoms, int m, int n_walkers, int K, ljh::Plan* out, b
     const size_t smem = bhc_head_bytes<T>(n_atoms) +
                         team_smem_bytes<T>(n_atoms, true, on_chip ? out->slot_bytes : 0);
     auto k = bh_cluster_kernel<T, A, MIXED, POT>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
     if (e != cudaSuccess) return e;
     if (K > 8) {
       e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);

@@ -165,12 +165,25 @@ __device__ __forceinline__ bool fisfinite(double a) { return isfinite(a); }
 __device__ __forceinline__ double fto_double(ff a) { return (double)a.hi + (double)a.lo; }
 __device__ __forceinline__ double fto_double(double a) { return a; }
 
+// s += v for a running double-float sum: TwoSum of the high words, every
+// rounding error and low word gathered in s.lo (Ogita, Rump and Oishi 2005,
+// Sum2); the chain of the high words is one addition a term.  s.lo is
+// renormalised where the sum is stored or scaled.
+__device__ __forceinline__ void df_acc(ff& s, ff v) {
+  const ff t = ff_two_sum(s.hi, v.hi);
+  s.hi = t.hi;
+  s.lo = __fadd_rn(s.lo, __fadd_rn(t.lo, v.lo));
+}
+
 template <int T>
 __device__ __forceinline__ ff team_sum_ff(const Team<T>& tm, ff v) {
+  // both partners of a butterfly step form the same sums: TwoSum's results
+  // and (v.lo + w.lo) do not depend on the order of the operands
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
-    ff w{shfl_xor(v.hi, o), shfl_xor(v.lo, o)};
-    v = ff_add(v, w);
+    const ff w{shfl_xor(v.hi, o), shfl_xor(v.lo, o)};
+    const ff t = ff_two_sum(v.hi, w.hi);
+    v = ff{t.hi, __fadd_rn(t.lo, __fadd_rn(v.lo, w.lo))};
   }
   if constexpr (T > 32) {
     constexpr int NW = T / 32;
@@ -182,35 +195,62 @@ __device__ __forceinline__ ff team_sum_ff(const Team<T>& tm, ff v) {
     tm.sync();
     ff s{buf[0], buf[1]};
 #pragma unroll
-    for (int w = 1; w < NW; ++w) s = ff_add(s, ff{buf[2 * w], buf[2 * w + 1]});
+    for (int w = 1; w < NW; ++w) df_acc(s, ff{buf[2 * w], buf[2 * w + 1]});
     v = s;
   }
   return v;
 }
 
-// team_sum of s[0..NS-1] and team_max of m[0..1] (inputs >= 0, non-finite
-// as +inf) in one pass, one cross-warp exchange; each value gets the
-// operations of its own reduction in the same order
-template <int T, typename V, typename M, int NS>
-__device__ __forceinline__ void team_sums_max2(const Team<T>& tm, V (&s)[NS], M (&m)[2]) {
+// Maximum of bit patterns over the team (bits of non-negative floats order as
+// integers): one or two REDUX instead of five shuffles with floating-point
+// maxima, which for FP64 each take the FP64 unit.
+__device__ __forceinline__ unsigned warp_max_bits(unsigned m) {
+  return __reduce_max_sync(kFull, m);
+}
+__device__ __forceinline__ unsigned long long warp_max_bits(unsigned long long m) {
+  const unsigned hi = (unsigned)(m >> 32);
+  const unsigned mh = __reduce_max_sync(kFull, hi);
+  const unsigned ml = __reduce_max_sync(kFull, hi == mh ? (unsigned)m : 0u);
+  return ((unsigned long long)mh << 32) | ml;
+}
+template <int T, typename B>
+__device__ __forceinline__ B team_max_bits(const Team<T>& tm, B m) {
+  m = warp_max_bits(m);
+  if constexpr (T > 32) {
+    constexpr int NW = T / 32;
+    B* buf = reinterpret_cast<B*>(tm.scratch());
+    if ((tm.rank & 31) == 0) buf[tm.rank >> 5] = m;
+    tm.sync();
+    m = buf[0];
+#pragma unroll
+    for (int w = 1; w < NW; ++w) m = max(m, buf[w]);
+  }
+  return m;
+}
+
+// team_sum of s[0..NS-1], the maximum of the bit patterns m and the
+// disjunction of f in one pass, one cross-warp exchange
+template <int T, typename V, typename B, int NS>
+__device__ __forceinline__ void team_sums_max(const Team<T>& tm, V (&s)[NS], B& m, bool& f) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
 #pragma unroll
     for (int k = 0; k < NS; ++k) s[k] += shfl_xor(s[k], o);
-#pragma unroll
-    for (int k = 0; k < 2; ++k) m[k] = fmax(m[k], shfl_xor(m[k], o));
   }
+  m = warp_max_bits(m);
+  f = __any_sync(kFull, f);
   if constexpr (T > 32) {
     constexpr int NW = T / 32;
-    static_assert(NS * sizeof(V) + 2 * sizeof(M) <= 8 * sizeof(double), "reduction scratch");
-    unsigned char* raw = reinterpret_cast<unsigned char*>(tm.scratch());
-    V* bs = reinterpret_cast<V*>(raw);
-    M* bm = reinterpret_cast<M*>(raw + ((NS * NW * sizeof(V) + sizeof(M) - 1) / sizeof(M)) * sizeof(M));
+    static_assert((NS + 1) * sizeof(V) + sizeof(B) + 8 <= 8 * sizeof(double), "reduction scratch");
+    double* raw = tm.scratch();
+    B* bm = reinterpret_cast<B*>(raw);
+    unsigned* bf = reinterpret_cast<unsigned*>(raw + NW);
+    V* bs = reinterpret_cast<V*>(raw + 2 * NW);
     if ((tm.rank & 31) == 0) {
 #pragma unroll
       for (int k = 0; k < NS; ++k) bs[(tm.rank >> 5) * NS + k] = s[k];
-#pragma unroll
-      for (int k = 0; k < 2; ++k) bm[(tm.rank >> 5) * 2 + k] = m[k];
+      bm[tm.rank >> 5] = m;
+      bf[tm.rank >> 5] = f;
     }
     tm.sync();
 #pragma unroll
@@ -220,13 +260,14 @@ __device__ __forceinline__ void team_sums_max2(const Team<T>& tm, V (&s)[NS], M 
       for (int w = 1; w < NW; ++w) a += bs[w * NS + k];
       s[k] = a;
     }
+    m = bm[0];
+    unsigned any = bf[0];
 #pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      M b = bm[k];
-#pragma unroll
-      for (int w = 1; w < NW; ++w) b = fmax(b, bm[w * 2 + k]);
-      m[k] = b;
+    for (int w = 1; w < NW; ++w) {
+      m = max(m, bm[w]);
+      any |= bf[w];
     }
+    f = any != 0;
   }
 }
 
@@ -236,9 +277,10 @@ template <int T>
 __device__ __forceinline__ void team_sum_ff_f(const Team<T>& tm, ff& e, float& x) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
-    ff w{shfl_xor(e.hi, o), shfl_xor(e.lo, o)};
-    e = ff_add(e, w);
+    const ff w{shfl_xor(e.hi, o), shfl_xor(e.lo, o)};
     x += shfl_xor(x, o);
+    const ff t = ff_two_sum(e.hi, w.hi);
+    e = ff{t.hi, __fadd_rn(t.lo, __fadd_rn(e.lo, w.lo))};
   }
   if constexpr (T > 32) {
     constexpr int NW = T / 32;
@@ -253,7 +295,7 @@ __device__ __forceinline__ void team_sum_ff_f(const Team<T>& tm, ff& e, float& x
     float t = buf[2];
 #pragma unroll
     for (int w = 1; w < NW; ++w) {
-      s = ff_add(s, ff{buf[3 * w], buf[3 * w + 1]});
+      df_acc(s, ff{buf[3 * w], buf[3 * w + 1]});
       t += buf[3 * w + 2];
     }
     e = s;
@@ -493,28 +535,32 @@ __device__ __forceinline__ void morse_row_f32x2(int n, int i, float px, float py
   bz = __fadd_rn(az.x, az.y);
 }
 
-// Double-double helpers: exact sum a + b = s + e (Knuth TwoSum).
 struct dd {
   double hi, lo;
 };
-__device__ __forceinline__ dd dd_two_sum(double a, double b) {
-  const double s = __dadd_rn(a, b);
-  const double bb = __dsub_rn(s, a);
-  const double e = __dadd_rn(__dsub_rn(a, __dsub_rn(s, bb)), __dsub_rn(b, bb));
-  return dd{s, e};
+// s += v for a running double-double sum (Sum2, as df_acc).  TwoSum with the
+// operands ordered by magnitude on the integer pipe: three FP64 additions
+// (Dekker's FastTwoSum) instead of six; a warp's FP64 instruction takes its
+// SM sub-partition's unit for 67 cycles.
+__device__ __forceinline__ void dd_acc(dd& s, dd v) {
+  const bool sw = (__double2hiint(s.hi) & 0x7fffffff) < (__double2hiint(v.hi) & 0x7fffffff);
+  const double a = sw ? v.hi : s.hi, b = sw ? s.hi : v.hi;
+  s.hi = __dadd_rn(a, b);
+  s.lo = __dadd_rn(__dsub_rn(b, __dsub_rn(s.hi, a)), __dadd_rn(s.lo, v.lo));
 }
-__device__ __forceinline__ dd dd_add(dd a, dd b) {
-  dd s = dd_two_sum(a.hi, b.hi);
-  return dd_two_sum(s.hi, __dadd_rn(s.lo, __dadd_rn(a.lo, b.lo)));
+__device__ __forceinline__ void dd_acc(dd& s, double v) {
+  const bool sw = (__double2hiint(s.hi) & 0x7fffffff) < (__double2hiint(v) & 0x7fffffff);
+  const double a = sw ? v : s.hi, b = sw ? s.hi : v;
+  s.hi = __dadd_rn(a, b);
+  s.lo = __dadd_rn(__dsub_rn(b, __dsub_rn(s.hi, a)), s.lo);
 }
 
 template <int T>
 __device__ __forceinline__ double team_sum_dd(const Team<T>& tm, dd v) {
+  // the error of a sum is the same number whichever operand FastTwoSum takes
+  // first, so both partners of a butterfly step hold the same bits
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    dd w{shfl_xor(v.hi, o), shfl_xor(v.lo, o)};
-    v = dd_add(v, w);
-  }
+  for (int o = 16; o > 0; o >>= 1) dd_acc(v, dd{shfl_xor(v.hi, o), shfl_xor(v.lo, o)});
   if constexpr (T > 32) {
     constexpr int NW = T / 32;
     double* buf = tm.scratch();
@@ -525,13 +571,13 @@ __device__ __forceinline__ double team_sum_dd(const Team<T>& tm, dd v) {
     tm.sync();
     dd s{buf[0], buf[1]};
 #pragma unroll
-    for (int w = 1; w < NW; ++w) s = dd_add(s, dd{buf[2 * w], buf[2 * w + 1]});
+    for (int w = 1; w < NW; ++w) dd_acc(s, dd{buf[2 * w], buf[2 * w + 1]});
     v = s;
   }
   return __dadd_rn(v.hi, v.lo);
 }
 
-// FP64: the reciprocal is the correctly rounded one; the energy is summed in
+// FP64: the energy is summed in
 // 4-term blocks folded into a compensated (double-double) accumulator, so
 // that near a minimum its rounding noise stays below the decreases the
 // line search must resolve (|E| ~ 170 for LJ38, decreases ~1e-12).
@@ -547,7 +593,7 @@ __device__ __forceinline__ void pair_row_f64(int n, int i, double px, double py,
       const PosD q = pos[j + u];
       const double dx = px - q.x, dy = py - q.y, dz = pz - q.z;
       const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
-      const double ir2 = (j + u == i) ? 0.0 : __drcp_rn(r2);
+      const double ir2 = (j + u == i) ? 0.0 : rcp_f64(r2);
       const double s2 = sig2 * ir2;
       const double s6 = s2 * s2 * s2;
       const double t = s6 - 1.0;
@@ -557,16 +603,14 @@ __device__ __forceinline__ void pair_row_f64(int n, int i, double px, double py,
       ay = fma(c, dy, ay);
       az = fma(c, dz, az);
     }
-    dd s = dd_two_sum(e.hi, eb);
-    e.hi = s.hi;
-    e.lo = __dadd_rn(e.lo, s.lo);
+    dd_acc(e, eb);
   }
   double eb = 0.0;
   for (; j < n; ++j) {
     const PosD q = pos[j];
     const double dx = px - q.x, dy = py - q.y, dz = pz - q.z;
     const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
-    const double ir2 = (j == i) ? 0.0 : __drcp_rn(r2);
+    const double ir2 = (j == i) ? 0.0 : rcp_f64(r2);
     const double s2 = sig2 * ir2;
     const double s6 = s2 * s2 * s2;
     const double t = s6 - 1.0;
@@ -576,9 +620,7 @@ __device__ __forceinline__ void pair_row_f64(int n, int i, double px, double py,
     ay = fma(c, dy, ay);
     az = fma(c, dz, az);
   }
-  dd s = dd_two_sum(e.hi, eb);
-  e.hi = s.hi;
-  e.lo = __dadd_rn(e.lo, s.lo);
+  dd_acc(e, eb);
 }
 
 // ---------------------------------------------------------------------------
@@ -609,6 +651,17 @@ __device__ __forceinline__ ff df_sub(ff a, ff b) {
   const ff s = ff_two_sum(a.hi, -b.hi);
   return df_fast_two_sum(s.hi, __fadd_rn(s.lo, __fsub_rn(a.lo, b.lo)));
 }
+// a - b and a b without the last renormalisation, for values that go into
+// df_norm2, a product or df_acc, which take an unnormalised pair: 8 and 4
+// operations instead of 11 and 7
+__device__ __forceinline__ ff df_sub_raw(ff a, ff b) {
+  const ff s = ff_two_sum(a.hi, -b.hi);
+  return ff{s.hi, __fadd_rn(s.lo, __fsub_rn(a.lo, b.lo))};
+}
+__device__ __forceinline__ ff df_mul_raw(ff a, ff b) {
+  const ff p = df_two_prod(a.hi, b.hi);
+  return ff{p.hi, fmaf(a.lo, b.hi, fmaf(a.hi, b.lo, p.lo))};
+}
 __device__ __forceinline__ ff df_add_f(ff a, float b) {
   const ff s = ff_two_sum(a.hi, b);
   return df_fast_two_sum(s.hi, __fadd_rn(s.lo, a.lo));
@@ -637,29 +690,21 @@ __device__ __forceinline__ ff df_from_double(double x) {
 }
 __device__ __forceinline__ double df_to_double(ff a) { return (double)a.hi + (double)a.lo; }
 
-// |d|^2 of a double-float vector with one renormalisation: the high squares
-// exactly (TwoProd by FMA), summed by two TwoSums, and every low-order part
-// (their rounding errors, 2 hi lo, the TwoProd errors) gathered in one FP32
-// word.  Dropped: lo^2 and the roundings of the low word, ~2^-47 relative.
+// |d|^2 of a double-float vector (not necessarily normalised) with one
+// renormalisation: the high squares exactly (TwoProd by FMA), summed by two
+// TwoSums, and every low-order part (their rounding errors, (2 hi + lo) lo, the
+// TwoProd errors) gathered in one FP32 word, whose roundings are ~2^-47 of the
+// result.
 __device__ __forceinline__ ff df_norm2(ff x, ff y, ff z) {
   const float px = __fmul_rn(x.hi, x.hi), py = __fmul_rn(y.hi, y.hi), pz = __fmul_rn(z.hi, z.hi);
   const float ex = fmaf(x.hi, x.hi, -px), ey = fmaf(y.hi, y.hi, -py), ez = fmaf(z.hi, z.hi, -pz);
   const ff s1 = ff_two_sum(px, py);
   const ff s2 = ff_two_sum(s1.hi, pz);
   float lo = __fadd_rn(__fadd_rn(s1.lo, s2.lo), __fadd_rn(__fadd_rn(ex, ey), ez));
-  lo = fmaf(__fadd_rn(x.hi, x.hi), x.lo, lo);
-  lo = fmaf(__fadd_rn(y.hi, y.hi), y.lo, lo);
-  lo = fmaf(__fadd_rn(z.hi, z.hi), z.lo, lo);
+  lo = fmaf(fmaf(2.f, x.hi, x.lo), x.lo, lo);
+  lo = fmaf(fmaf(2.f, y.hi, y.lo), y.lo, lo);
+  lo = fmaf(fmaf(2.f, z.hi, z.lo), z.lo, lo);
   return df_fast_two_sum(s2.hi, lo);
-}
-
-// s += v for a running double-float sum: TwoSum of the high words, every
-// rounding error and low word gathered in s.lo (Ogita, Rump and Oishi 2005,
-// Sum2); s.lo is renormalised where the sum is stored
-__device__ __forceinline__ void df_acc(ff& s, ff v) {
-  const ff t = ff_two_sum(s.hi, v.hi);
-  s.hi = t.hi;
-  s.lo = __fadd_rn(s.lo, __fadd_rn(t.lo, v.lo));
 }
 
 // sqrt(a) in double-float (Karp and Markstein, ACM TOMS 1997): y ~ 1/sqrt(a)
@@ -721,15 +766,15 @@ __device__ __forceinline__ ff df_exp(ff x) {
 // (+inf for coincident atoms).  rho is the double-float range parameter.
 __device__ __forceinline__ void pair_term_morse_df(const PosDF& a, const PosDF& b, ff rho,
                                                    ff& vx, ff& vy, ff& vz, ff& e) {
-  const ff dx = df_sub(ff{a.xh, a.xl}, ff{b.xh, b.xl});
-  const ff dy = df_sub(ff{a.yh, a.yl}, ff{b.yh, b.yl});
-  const ff dz = df_sub(ff{a.zh, a.zl}, ff{b.zh, b.zl});
+  const ff dx = df_sub_raw(ff{a.xh, a.xl}, ff{b.xh, b.xl});
+  const ff dy = df_sub_raw(ff{a.yh, a.yl}, ff{b.yh, b.yl});
+  const ff dz = df_sub_raw(ff{a.zh, a.zl}, ff{b.zh, b.zl});
   const ff r2 = df_norm2(dx, dy, dz);
   const ff r = df_sqrt(r2);
   const ff ex = df_exp(df_sub(rho, df_mul(rho, r)));
   e = r2.hi > 0.f ? df_mul(ex, df_add_f(ex, -2.f)) : ff{__int_as_float(0x7f800000), 0.f};
   const ff c = df_mul(df_mul(ex, df_add_f(ex, -1.f)), df_rcp(r));
-  vx = df_mul(c, dx); vy = df_mul(c, dy); vz = df_mul(c, dz);
+  vx = df_mul_raw(c, dx); vy = df_mul_raw(c, dy); vz = df_mul_raw(c, dz);
 }
 
 // One row of the pair sum in df arithmetic, coordinates pre-scaled by
@@ -759,43 +804,109 @@ __device__ __forceinline__ void pair_row_df(int n, int i, ff px, ff py, ff pz,
 }
 
 // ---------------------------------------------------------------------------
-// Half-pair evaluation (FP64 and double-float): each unordered pair i < j is
-// computed once, by thread (p mod T) of the team, p the pair's index in
-// row-major order of the upper triangle; its vector v_p = c_ij (x_i - x_j)
-// goes to a shared buffer, and after a barrier the thread owning atom i sums
-// +v over j > i and -v over j < i.  Every pair costs one evaluation instead
-// of two (the one-sided loop visits it from both atoms) and the work splits
-// evenly over the team whatever N is -- for N = 38 on a warp, 22 pairs per
-// thread instead of 74.  Deterministic: fixed pair order, fixed sum order.
+// Half-pair evaluation (FP64 and double-float, clusters of up to 64 atoms):
+// each unordered pair once, in the order of a ring: pair p is atom i = p mod n
+// with j = (i + k) mod n, k = 1 + p / n (for even n the shift n/2 holds the n/2
+// pairs i < n/2).  Thread p mod T evaluates it and writes its vector
+// v_p = c_ij (x_i - x_j) to a shared buffer; after a barrier the sum of an atom
+// and axis takes +v of the pairs that start at the atom, ((k-1) n + atom), and
+// -v of those that end there, ((k-1) n + (atom - k) mod n).  Both run through
+// the buffer with consecutive lanes at consecutive words: no bank conflicts and
+// one index and one comparison a term, where the triangular order took a
+// select of two row bases, a select of the sign and eight-byte strides of a
+// whole row.  Every pair costs one evaluation instead of two and the work
+// splits evenly over the team whatever N is.  Fixed pair order, fixed sum order.
 // ---------------------------------------------------------------------------
 __host__ __device__ constexpr int n_pairs(int n) { return n * (n - 1) / 2; }
 
-// index of pair (i, j), i < j, in the row-major upper triangle
-__device__ __forceinline__ int pair_index(int n, int i, int j) {
-  return i * (2 * n - i - 1) / 2 + (j - i - 1);
+// pair (i, j) of index p, advanced by a fixed step
+struct PairWalk {
+  int i, k;
+  __device__ __forceinline__ PairWalk(int n, int p) : i(p % n), k(1 + p / n) {}
+  __device__ __forceinline__ int j(int n) const {
+    const int t = i + k;
+    return t >= n ? t - n : t;
+  }
+  // step = dk n + di, 0 <= di < n
+  __device__ __forceinline__ void advance(int n, int dk, int di) {
+    i += di;
+    k += dk;
+    if (i >= n) { i -= n; ++k; }
+  }
+};
+
+// two pairs in flight a thread (the second clamped to pair (0, 1) past the end
+// and discarded); term(i, j, vx, vy, vz, e) evaluates one, add(e) takes its
+// energy
+template <int T, typename F, typename Term, typename Add>
+__device__ __forceinline__ void half_pairs(int rank, int n, F* vb, Term&& term, Add&& add) {
+  const int np = n_pairs(n);
+  const int dk = 2 * T / n, di = 2 * T - dk * n;
+  PairWalk w1(n, rank), w2(n, rank + T);
+  for (int q = rank; q < np; q += 2 * T) {
+    const bool two = q + T < np;
+    F ax, ay, az, ae, bx, by, bz, be;
+    term(w1.i, w1.j(n), ax, ay, az, ae);
+    term(two ? w2.i : 0, two ? w2.j(n) : 1, bx, by, bz, be);
+    vb[q] = ax; vb[np + q] = ay; vb[2 * np + q] = az;
+    add(ae);
+    if (two) {
+      vb[q + T] = bx; vb[np + q + T] = by; vb[2 * np + q + T] = bz;
+      add(be);
+    }
+    w1.advance(n, dk, di);
+    w2.advance(n, dk, di);
+  }
 }
 
-// pair_index(n, a, b) = row_base(n, a) + b, so that pair (j, i), j < i, sits at
-// row_base(n, j) + i and pair (i, j), j > i, at row_base(n, i) + j;
-// row_base(n, j + 1) = row_base(n, j) + n - j - 2, row_base(n, 0) = -1
-__device__ __forceinline__ int row_base(int n, int i) {
-  return i * (2 * n - i - 1) / 2 - i - 1;
+__device__ __forceinline__ void half_plus(ff& s, ff v) { df_acc(s, v); }
+__device__ __forceinline__ void half_minus(ff& s, ff v) { df_acc(s, ff{-v.hi, -v.lo}); }
+__device__ __forceinline__ float half_total(ff a, ff b, ff c, ff d) {
+  df_acc(a, c); df_acc(b, d); df_acc(a, b);
+  return __fadd_rn(a.hi, a.lo);
+}
+__device__ __forceinline__ void half_plus(double& s, double v) { s += v; }
+__device__ __forceinline__ void half_minus(double& s, double v) { s -= v; }
+__device__ __forceinline__ double half_total(double a, double b, double c, double d) {
+  return (a + c) + (b + d);              // the pairs that start, then those that end
 }
 
-// first pair (i, j) of thread `rank` (p = rank); -1 if none
-__device__ __forceinline__ void pair_start(int n, int p, int& i, int& j) {
-  i = 0;
-  int row = n - 1;
-  while (row > 0 && p >= row) { p -= row; ++i; --row; }
-  j = row > 0 ? i + 1 + p : -1;
-}
-// advance (i, j) by `step` pairs
-__device__ __forceinline__ void pair_advance(int n, int step, int& i, int& j) {
-  j += step;
-  while (i < n - 1 && j >= n) {
-    j -= n;         // j - n = offset past the row end
-    ++i;
-    j += i + 1;     // first column of the next row is i+1
+// sums[3 atom + axis] = scale * sum, one (axis, atom) a thread, four
+// independent sums each
+template <int T, typename F, typename G>
+__device__ __forceinline__ void half_rows(int rank, int n, const F* vb, G scale, G* sums) {
+  const int np = n_pairs(n), H = (n - 1) >> 1;
+  for (int q3 = rank; q3 < 3 * n; q3 += T) {
+    const int axis = q3 >= 2 * n ? 2 : q3 >= n ? 1 : 0;
+    const int ii = q3 - axis * n;
+    const F* vc = vb + axis * np;
+    const F* vp = vc + ii;                 // pairs that start at the atom
+    int e = ii;                            // (atom - k) mod n
+    F s0{}, s1{}, s2{}, s3{};
+    int k = 0;
+    for (; k + 2 <= H; k += 2) {
+      const int e1 = e > 0 ? e - 1 : n - 1;
+      const int e2 = e1 > 0 ? e1 - 1 : n - 1;
+      const F a = vp[0], b = vc[e1], c = vp[n], d = vc[n + e2];
+      half_plus(s0, a);
+      half_minus(s1, b);
+      half_plus(s2, c);
+      half_minus(s3, d);
+      e = e2;
+      vp += 2 * n;
+      vc += 2 * n;
+    }
+    if (k < H) {
+      half_plus(s0, vp[0]);
+      half_minus(s1, vc[e > 0 ? e - 1 : n - 1]);
+      vp += n;
+      vc += n;
+    }
+    if (!(n & 1)) {                        // the half shift of an even n
+      if (ii < n / 2) half_plus(s2, vp[0]);
+      else half_minus(s3, vc[ii - n / 2]);
+    }
+    sums[3 * ii + axis] = scale * half_total(s0, s1, s2, s3);
   }
 }
 
@@ -804,7 +915,7 @@ __device__ __forceinline__ void pair_term_f64(const PosD& a, const PosD& b, doub
                                               double& vx, double& vy, double& vz, double& e) {
   const double dx = a.x - b.x, dy = a.y - b.y, dz = a.z - b.z;
   const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
-  const double s2 = sig2 * __drcp_rn(r2);
+  const double s2 = sig2 * rcp_f64(r2);
   const double s6 = s2 * s2 * s2;
   const double t = s6 - 1.0;
   e = s6 * t;
@@ -812,19 +923,80 @@ __device__ __forceinline__ void pair_term_f64(const PosD& a, const PosD& b, doub
   vx = c * dx; vy = c * dy; vz = c * dz;
 }
 
-// pair term in double-float on coordinates scaled by 1/sigma
+// pair term in double-float on coordinates scaled by 1/sigma: with s12 = s6^2,
+// e = s12 - s6 and c = s2 (s12 + e).  v and e are not renormalised (they are
+// summed by df_acc).  123 FP32 operations.
 __device__ __forceinline__ void pair_term_df(const PosDF& a, const PosDF& b, ff& vx, ff& vy,
                                              ff& vz, ff& e) {
-  const ff dx = df_sub(ff{a.xh, a.xl}, ff{b.xh, b.xl});
-  const ff dy = df_sub(ff{a.yh, a.yl}, ff{b.yh, b.yl});
-  const ff dz = df_sub(ff{a.zh, a.zl}, ff{b.zh, b.zl});
+  const ff dx = df_sub_raw(ff{a.xh, a.xl}, ff{b.xh, b.xl});
+  const ff dy = df_sub_raw(ff{a.yh, a.yl}, ff{b.yh, b.yl});
+  const ff dz = df_sub_raw(ff{a.zh, a.zl}, ff{b.zh, b.zl});
   const ff r2 = df_norm2(dx, dy, dz);
   const ff s2 = df_rcp(r2);
   const ff s6 = df_mul(df_sqr(s2), s2);
-  const ff t = df_add_f(s6, -1.f);
-  e = df_mul(s6, t);
-  const ff c = df_mul(df_mul(s2, s6), df_add(s6, t));
-  vx = df_mul(c, dx); vy = df_mul(c, dy); vz = df_mul(c, dz);
+  const ff s12 = df_sqr(s6);
+  e = df_sub_raw(s12, s6);
+  const ff c = df_mul(s2, df_add(s12, e));
+  vx = df_mul_raw(c, dx); vy = df_mul_raw(c, dy); vz = df_mul_raw(c, dz);
+}
+
+// ---------------------------------------------------------------------------
+// Ring evaluation (FP64 and double-float, clusters of 65 to 256 atoms): every
+// unordered pair once, by the thread of atom i at shift k with j = (i + k) mod
+// n, k = 1 .. n/2 (at k = n/2 of an even n, i < n/2 only).  The thread adds
+// v = c (x_i - x_j) to its own atom in registers and leaves it for j in the
+// buffer (KS shifts of n entries, one writer each); after a barrier the owners
+// subtract, in the order of the shifts.  Two pairs in flight a thread.
+// ---------------------------------------------------------------------------
+template <int T, int A, typename F, typename Term, typename Add>
+__device__ __forceinline__ void ring_pairs(const Team<T>& tm, int n, int KS, F* buf, Term&& term,
+                                           Add&& add, F (&acc)[A][3]) {
+  const int full = (n - 1) >> 1;           // shifts that every atom takes
+  const int last = n >> 1;                 // > full: the half shift
+#pragma unroll
+  for (int a = 0; a < A; ++a)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) acc[a][c] = F{};
+  auto one = [&](int a, int i, int k, F* b) {
+    int j = i + k;
+    if (j >= n) j -= n;
+    F vx, vy, vz, e;
+    term(i, j, vx, vy, vz, e);
+    half_plus(acc[a][0], vx);
+    half_plus(acc[a][1], vy);
+    half_plus(acc[a][2], vz);
+    add(e);
+    b[j] = vx; b[n + j] = vy; b[2 * n + j] = vz;
+  };
+  for (int k0 = 1; k0 <= last; k0 += KS) {
+    const int ks = min(KS, last - k0 + 1);
+    if (k0 > 1) tm.sync();                 // the last chunk's readers are done
+    const int nf = min(ks, full - k0 + 1);
+#pragma unroll
+    for (int a = 0; a < A; ++a) {
+      const int i = tm.rank + a * T;
+      if (i < n) {
+        int s = 0;
+        for (; s + 2 <= nf; s += 2) {
+          one(a, i, k0 + s, buf + 3 * n * s);
+          one(a, i, k0 + s + 1, buf + 3 * n * (s + 1));
+        }
+        if (s < nf) one(a, i, k0 + s, buf + 3 * n * s);
+        if (nf < ks && i < last) one(a, i, last, buf + 3 * n * nf);
+      }
+    }
+    tm.sync();
+#pragma unroll
+    for (int a = 0; a < A; ++a) {
+      const int i = tm.rank + a * T;
+      if (i < n) {
+        const int ns = nf < ks && i >= last ? ks : nf;
+        for (int s = 0; s < ns; ++s)
+#pragma unroll
+          for (int c = 0; c < 3; ++c) half_minus(acc[a][c], buf[3 * n * s + c * n + i]);
+      }
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -969,9 +1141,7 @@ __device__ void d_tile_eval(const Team<T>& tm, int n, const PosD* __restrict__ p
       hy = __shfl_sync(kFull, hy, src);
       hz = __shfl_sync(kFull, hz, src);
     }
-    const dd t = dd_two_sum(e.hi, eb);
-    e.hi = t.hi;
-    e.lo = __dadd_rn(e.lo, t.lo);
+    dd_acc(e, eb);
     if (diag) {
       fx += hx; fy += hy; fz += hz;
     } else if (jl < n) {

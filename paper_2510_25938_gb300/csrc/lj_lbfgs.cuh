@@ -19,16 +19,27 @@ __device__ __forceinline__ MinParams to_dev(const ljh::MinParamsH& h) {
   p.gtol = h.gtol; p.c1 = h.c1; p.c2 = h.c2; p.alpha_max = h.alpha_max;
   p.switch_gtol = h.switch_gtol; p.deadline = h.deadline; p.k = h.k;
   p.f32_resolution = h.f32_resolution; p.df_resolution = h.df_resolution;
-  p.tiled = 0;
+  p.layout = 0;
+  p.ring_ks = 1;
   return p;
 }
 
-// Register budget: teams for more than 256 atoms (which carry the tiled
-// double-float evaluation) are allowed all registers of one CTA per SM; the
-// others are left to the compiler's own occupancy choice.
+// Register budget.  Mixed precision, teams of up to 64 threads: two CTAs of 128
+// threads an SM, 255 registers; left to itself the compiler stops at 168 with
+// spills, and the third CTA that this leaves room for does not make up for them
+// (4,096 x LJ38: 2.64 against 2.82 ms).  128 threads with one atom each: three
+// CTAs; their ring evaluation waits for its own chains, and a third CTA hides
+// more of that than 168 registers cost (1,024 x 100 atoms: 4.24 against 4.66
+// ms).  256 threads with two atoms each: two CTAs, 128 registers; the tiled
+// evaluation is bound by latency with eight warps an SM, and sixteen pay for
+// its spills (1,024 x 500 atoms, mixed: 71.2 against 79.7 ms).  512 threads:
+// all registers of one CTA.
 // POT: pair potential (LJ_POT_LJ, Eq. (1); LJ_POT_MORSE).
+constexpr int min_ctas(int T, int A, bool mixed) {
+  return mixed && T <= 64 ? 2 : mixed && T * A <= 128 ? 3 : T * A <= 256 ? 0 : T == 256 ? 2 : 1;
+}
 template <int T, int A, bool MIXED, int POT = LJ_POT_LJ>
-__global__ void __launch_bounds__(cta_threads_for(T), T * A > 256 ? 1 : 0)
+__global__ void __launch_bounds__(cta_threads_for(T), min_ctas(T, A, MIXED))
     lbfgs_kernel(ljh::LbfgsArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int TPC = cta_threads_for(T) / T;
@@ -44,11 +55,12 @@ __global__ void __launch_bounds__(cta_threads_for(T), T * A > 256 ? 1 : 0)
   carve_team<T>(smem + team * team_smem_bytes<T>(a.max_n, true, hb), a.max_n, true, hb, pos,
                 hbuf, hist, tm.red, word);
   MinParams p = to_dev(a.p);
-  // hbuf: pair buffer up to 64 atoms, tile accumulators above 256.  With
+  // hbuf: pairs up to 64 atoms, ring chunks up to 256, tile accumulators above.  With
   // one-sided rows chosen above 256 atoms there is no pair buffer to use: the
   // buffer holds 24 bytes per atom, not per pair, so it is withdrawn and every
   // tier evaluates in one-sided rows
-  p.tiled = a.max_n > kTileMinN && !a.p.df_one_sided;
+  p.layout = pair_layout(a.max_n);
+  p.ring_ks = ring_shifts(a.max_n);
   if (a.max_n > kTileMinN && a.p.df_one_sided) hbuf = nullptr;
   const long long slot = (long long)blockIdx.x * TPC + team;
   if (!a.hist_on_chip) hist = static_cast<unsigned char*>(a.hist) + slot * a.hist_slot_bytes;
@@ -145,7 +157,7 @@ cudaError_t plan_one(int max_n, int m, int64_t n_cand, int device, ljh::Plan* ou
       !hist_global && TPC * team_smem_bytes<T>(max_n, true, hist_bytes) <= kSmemBudget;
   const size_t smem = TPC * team_smem_bytes<T>(max_n, true, on_chip ? hist_bytes : 0);
   auto k = lbfgs_kernel<T, A, MIXED, POT>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
   if (e != cudaSuccess) return e;
   int sms = 0, per_sm = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);

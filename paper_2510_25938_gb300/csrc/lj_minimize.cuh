@@ -35,6 +35,7 @@
 #include <type_traits>
 
 #include "lj_device.cuh"
+#include "lj_teams.cuh"
 #include "lj_consts.h"
 #include "../../include/lj_bh.h"
 
@@ -45,7 +46,8 @@ struct MinParams {
   double gtol, c1, c2, alpha_max, switch_gtol;
   long long deadline;
   ljh::LjConsts k;         // pair-potential constants (host-derived)
-  int tiled;               // hbuf holds tile accumulators (teams for > 64 atoms), not pairs
+  int layout;              // what hbuf holds (PairLayout)
+  int ring_ks;             // ... its ring chunk, in shifts
   double f32_resolution;   // FP32 phase hands over below this predicted decrease / |E|
   double df_resolution;    // double-float polish hands over below this / |E|
 };
@@ -112,13 +114,18 @@ template <typename V> __device__ __forceinline__ V eps_mach();
 template <> __device__ __forceinline__ float eps_mach<float>() { return 1.1920928955078125e-7f; }
 template <> __device__ __forceinline__ double eps_mach<double>() { return 2.220446049250313e-16; }
 
+__device__ __forceinline__ float recip(float x) { return __frcp_rn(x); }
+__device__ __forceinline__ double recip(double x) { return rcp_f64(x); }
 __device__ __forceinline__ float S_sqrt(float x) { return sqrtf(x); }
 __device__ __forceinline__ double S_sqrt(double x) { return sqrt(x); }
 
-// history element (slot, atom slot a, component c) of this thread
+// history element (slot, atom slot a, component c) of this thread: a slot is
+// the flattened 3N vector for teams whose first warp runs the recursion (it
+// reads 16 bytes a lane), one plane per (a, c) above
 template <int T, int A>
 __device__ __forceinline__ int hidx(int slot, int a, int c, int rank) {
-  return ((slot * A + a) * 3 + c) * T + rank;
+  if constexpr (T <= 128) return (slot * A * T + a * T + rank) * 3 + c;
+  else return ((slot * A + a) * 3 + c) * T + rank;
 }
 
 // ---------------------------------------------------------------------------
@@ -142,15 +149,33 @@ __device__ __forceinline__ int hidx(int slot, int a, int c, int rank) {
 // then every (atom, component) row is summed, +v over j > i, -v over j < i.
 // Coincident atoms give E = +inf (and a non-finite gradient), as for Eq. (1).
 // ---------------------------------------------------------------------------
+__device__ __forceinline__ float to_value(ff v) { return v.hi + v.lo; }
+__device__ __forceinline__ double to_value(double v) { return v; }
+
+// gradient of the owned atoms from the ring's sums, and this thread's g.d
+template <int T, int A, typename P, typename F, typename G>
+__device__ __forceinline__ void ring_gradient(const Team<T>& tm, int n, const F (&acc)[A][3],
+                                              G scale, typename P::XG (&g)[A][3],
+                                              const typename P::V (*d)[3], typename P::V& dp) {
+  using V = typename P::V;
+#pragma unroll
+  for (int a = 0; a < A; ++a) {
+    const bool in = tm.rank + a * T < n;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) g[a][c] = in ? scale * to_value(acc[a][c]) : (typename P::XG)0;
+    if (d) dp += (V)g[a][0] * d[a][0] + (V)g[a][1] * d[a][1] + (V)g[a][2] * d[a][2];
+  }
+}
+
 __device__ __forceinline__ void pair_term_morse_f64(const PosD& a, const PosD& b, double rho,
                                                     double rr, double& vx, double& vy,
                                                     double& vz, double& e) {
   const double dx = a.x - b.x, dy = a.y - b.y, dz = a.z - b.z;
   const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
-  const double r = sqrt(r2);
-  const double ex = exp(fma(-rr, r, rho));
+  const double ir = rsqrt_f64(r2);
+  const double ex = exp(fma(-rr, r2 * ir, rho));
   e = r2 > 0.0 ? ex * (ex - 2.0) : __longlong_as_double(0x7ff0000000000000LL);
-  const double c = ex * (ex - 1.0) / r;
+  const double c = ex * (ex - 1.0) * ir;
   vx = c * dx; vy = c * dy; vz = c * dz;
 }
 
@@ -186,53 +211,16 @@ __device__ __forceinline__ void evaluate_morse_df(const Team<T>& tm, int n,
   const float gs = p.k.m_g_f;
   V dp = (V)0;
   ff e{0.f, 0.f};
-  if (hbuf != nullptr && !p.tiled) {
-    const int np = n_pairs(n);
+  if (hbuf != nullptr && p.layout == LAYOUT_HALF) {
     ff* vb = static_cast<ff*>(hbuf);
     float* gsum = static_cast<float*>(posv);
-    int i1, j1, i2, j2;
-    pair_start(n, tm.rank, i1, j1);
-    i2 = i1; j2 = j1;
-    pair_advance(n, T, i2, j2);
-    for (int q = tm.rank; q < np; q += 2 * T) {
-      const bool two = q + T < np;
-      const int ib = two ? i2 : 0, jb = two ? j2 : 1;
-      ff ax, ay, az, ae, bx, by, bz, be;
-      pair_term_morse_df(pos[i1], pos[j1], rho, ax, ay, az, ae);
-      pair_term_morse_df(pos[ib], pos[jb], rho, bx, by, bz, be);
-      vb[q] = ax; vb[np + q] = ay; vb[2 * np + q] = az;
-      df_acc(e, ae);
-      if (two) {
-        vb[q + T] = bx; vb[np + q + T] = by; vb[2 * np + q + T] = bz;
-        df_acc(e, be);
-      }
-      pair_advance(n, 2 * T, i1, j1);
-      pair_advance(n, 2 * T, i2, j2);
-    }
+    half_pairs<T>(tm.rank, n, vb,
+                  [&](int i, int j, ff& vx, ff& vy, ff& vz, ff& ep) {
+                    pair_term_morse_df(pos[i], pos[j], rho, vx, vy, vz, ep);
+                  },
+                  [&](ff ep) { df_acc(e, ep); });
     tm.sync();
-    for (int q3 = tm.rank; q3 < 3 * n; q3 += T) {
-      const int ii = q3 / 3;
-      const ff* vc = vb + (q3 - 3 * ii) * np;
-      const int ri = row_base(n, ii);       // all lanes walk j together
-      int rj = -1;
-      ff sacc[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
-      for (int j0 = 0; j0 < n; j0 += 4) {
-        ff v[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int j = j0 + u;
-          const int qq = j < ii ? rj + ii : ri + j;
-          v[u] = ff{0.f, 0.f};
-          if (j < n && j != ii) v[u] = vc[qq];
-          if (j < ii) v[u] = ff{-v[u].hi, -v[u].lo};
-          rj += n - j - 2;
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) df_acc(sacc[u], v[u]);
-      }
-      const ff sum = df_add(df_add(sacc[0], sacc[1]), df_add(sacc[2], sacc[3]));
-      gsum[q3] = -gs * (sum.hi + sum.lo);
-    }
+    half_rows<T>(tm.rank, n, vb, -gs, gsum);
     tm.sync();
 #pragma unroll
     for (int a = 0; a < A; ++a) {
@@ -244,6 +232,15 @@ __device__ __forceinline__ void evaluate_morse_df(const Team<T>& tm, int n,
       }
       if (d) dp += (V)g[a][0] * d[a][0] + (V)g[a][1] * d[a][1] + (V)g[a][2] * d[a][2];
     }
+    E = ff_scale(team_sum_ff<T>(tm, e), p.k.eps_f);
+  } else if (T * A <= 256 && hbuf != nullptr && p.layout == LAYOUT_RING) {
+    ff acc[A][3];
+    ring_pairs<T, A>(tm, n, p.ring_ks, static_cast<ff*>(hbuf),
+                     [&](int i, int j, ff& vx, ff& vy, ff& vz, ff& ep) {
+                       pair_term_morse_df(pos[i], pos[j], rho, vx, vy, vz, ep);
+                     },
+                     [&](ff ep) { df_acc(e, ep); }, acc);
+    ring_gradient<T, A, P>(tm, n, acc, -gs, g, d, dp);
     E = ff_scale(team_sum_ff<T>(tm, e), p.k.eps_f);
   } else {
 #pragma unroll
@@ -333,60 +330,20 @@ __device__ __forceinline__ void evaluate_morse(const Team<T>& tm, int n,
       }
     }
     E = ff_scale(team_sum_ff<T>(tm, e), p.k.m_half_f);
-  } else if (hbuf != nullptr && !p.tiled) {
+  } else if (hbuf != nullptr && p.layout == LAYOUT_HALF) {
     // ---- half-pair FP64 evaluation (pair phase, then row sums) -------------
-    const int np = n_pairs(n);
     const PosD* pos = static_cast<const PosD*>(posv);
     double* vb = static_cast<double*>(hbuf);
     double* gsum = static_cast<double*>(posv);
     const double rho = p.k.rho, rr = p.k.rho_re;
-    int i1, j1, i2, j2;
-    pair_start(n, tm.rank, i1, j1);
-    i2 = i1; j2 = j1;
-    pair_advance(n, T, i2, j2);
     dd e{0.0, 0.0};
-    for (int q = tm.rank; q < np; q += 2 * T) {
-      const bool two = q + T < np;
-      const int ib = two ? i2 : 0, jb = two ? j2 : 1;
-      double ax, ay, az, ae, bx, by, bz, be;
-      pair_term_morse_f64(pos[i1], pos[j1], rho, rr, ax, ay, az, ae);
-      pair_term_morse_f64(pos[ib], pos[jb], rho, rr, bx, by, bz, be);
-      vb[q] = ax; vb[np + q] = ay; vb[2 * np + q] = az;
-      double eb = ae;
-      if (two) {
-        vb[q + T] = bx; vb[np + q + T] = by; vb[2 * np + q + T] = bz;
-        eb += be;
-      }
-      const dd t = dd_two_sum(e.hi, eb);    // compensated energy sum
-      e.hi = t.hi;
-      e.lo = __dadd_rn(e.lo, t.lo);
-      pair_advance(n, 2 * T, i1, j1);
-      pair_advance(n, 2 * T, i2, j2);
-    }
+    half_pairs<T>(tm.rank, n, vb,
+                  [&](int i, int j, double& vx, double& vy, double& vz, double& ep) {
+                    pair_term_morse_f64(pos[i], pos[j], rho, rr, vx, vy, vz, ep);
+                  },
+                  [&](double ep) { dd_acc(e, ep); });   // compensated energy sum
     tm.sync();
-    const double gs = p.k.m_g;
-    for (int q3 = tm.rank; q3 < 3 * n; q3 += T) {
-      const int ii = q3 / 3;
-      const double* vc = vb + (q3 - 3 * ii) * np;
-      const int ri = row_base(n, ii);       // all lanes walk j together
-      int rj = -1;
-      double sacc[4] = {0.0, 0.0, 0.0, 0.0};
-      for (int j0 = 0; j0 < n; j0 += 4) {
-        double v[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int j = j0 + u;
-          const int qq = j < ii ? rj + ii : ri + j;
-          v[u] = 0.0;
-          if (j < n && j != ii) v[u] = vc[qq];
-          if (j < ii) v[u] = -v[u];
-          rj += n - j - 2;
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) sacc[u] += v[u];
-      }
-      gsum[q3] = -gs * ((sacc[0] + sacc[1]) + (sacc[2] + sacc[3]));
-    }
+    half_rows<T>(tm.rank, n, vb, -p.k.m_g, gsum);
     tm.sync();
 #pragma unroll
     for (int a = 0; a < A; ++a) {
@@ -399,6 +356,18 @@ __device__ __forceinline__ void evaluate_morse(const Team<T>& tm, int n,
       if (d) dp += (V)g[a][0] * d[a][0] + (V)g[a][1] * d[a][1] + (V)g[a][2] * d[a][2];
     }
     E = team_sum_dd<T>(tm, e) * p.k.eps;
+  } else if (T * A <= 256 && hbuf != nullptr && p.layout == LAYOUT_RING) {
+    const PosD* pos = static_cast<const PosD*>(posv);
+    const double rho = p.k.rho, rr = p.k.rho_re;
+    double acc[A][3];
+    dd e{0.0, 0.0};
+    ring_pairs<T, A>(tm, n, p.ring_ks, static_cast<double*>(hbuf),
+                     [&](int i, int j, double& vx, double& vy, double& vz, double& ep) {
+                       pair_term_morse_f64(pos[i], pos[j], rho, rr, vx, vy, vz, ep);
+                     },
+                     [&](double ep) { dd_acc(e, ep); }, acc);
+    ring_gradient<T, A, P>(tm, n, acc, -p.k.m_g, g, d, dp);
+    E = team_sum_dd<T>(tm, e) * p.k.eps;
   } else {
     const Q* pos = static_cast<const Q*>(posv);
     const double rho = p.k.rho, rr = p.k.rho_re, gsc = p.k.m_g;
@@ -410,31 +379,25 @@ __device__ __forceinline__ void evaluate_morse(const Team<T>& tm, int n,
       if (i < n) {
         const double xi = x[a][0], yi = x[a][1], zi = x[a][2];
         double ax = 0.0, ay = 0.0, az = 0.0;
-        double eb = 0.0;
         for (int j = 0; j < n; ++j) {
           const Q q = pos[j];
           const double dx = xi - q.x, dy = yi - q.y, dz = zi - q.z;
           const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
-          const double r = sqrt(r2);
-          const double ex = exp(fma(-rr, r, rho));
+          const double ir = rsqrt_f64(r2);
+          const double ex = exp(fma(-rr, r2 * ir, rho));
           double term = ex * (ex - 2.0);
-          double c = ex * (ex - 1.0) / r;
+          double c = ex * (ex - 1.0) * ir;
           if (j == i) {
             term = 0.0;
             c = 0.0;
           } else if (!(r2 > 0.0)) {
             term = kInf;
           }
-          const dd t = dd_two_sum(eb, term);      // compensated row energy
-          eb = t.hi;
-          e.lo = __dadd_rn(e.lo, t.lo);
+          dd_acc(e, term);                        // compensated energy
           ax = fma(c, dx, ax);
           ay = fma(c, dy, ay);
           az = fma(c, dz, az);
         }
-        const dd t = dd_two_sum(e.hi, eb);
-        e.hi = t.hi;
-        e.lo = __dadd_rn(e.lo, t.lo);
         g[a][0] = -gsc * ax; g[a][1] = -gsc * ay; g[a][2] = -gsc * az;
       } else {
         g[a][0] = 0.0; g[a][1] = 0.0; g[a][2] = 0.0;
@@ -488,126 +451,34 @@ __device__ __forceinline__ void evaluate(const Team<T>& tm, int n,
   V dp = (V)0;
   if constexpr (PM == 1 || std::is_same<X, double>::value) {
     ff e_df{0.f, 0.f};          // PM == 1: this thread's pair energies
-    if (hbuf != nullptr && !p.tiled) {
-      // ---- half-pair evaluation ---------------------------------------------
-      // pair phase: thread `rank` takes pairs rank, rank + T, ...; two pairs
-      // per iteration (the second one clamped to a valid pair and discarded
-      // past the end) keep two independent dependency chains in flight.
-      // sum phase: one (atom, component) row sum per thread, written over the
-      // position buffer (no longer needed), then read back by the owners.
-      const int np = n_pairs(n);
-      int i1, j1, i2, j2;
-      pair_start(n, tm.rank, i1, j1);
-      i2 = i1; j2 = j1;
-      pair_advance(n, T, i2, j2);
+    if (hbuf != nullptr && p.layout == LAYOUT_HALF) {
+      // ---- half-pair evaluation: pairs, then one (atom, axis) sum a thread,
+      // written over the position buffer (no longer needed) and read back by
+      // the owners
       XG* gsum = static_cast<XG*>(posv);
       if constexpr (PM == 1) {
         const PosDF* pos = static_cast<const PosDF*>(posv);
         ff* vb = static_cast<ff*>(hbuf);
-        ff e{0.f, 0.f};
-        for (int q = tm.rank; q < np; q += 2 * T) {
-          const bool two = q + T < np;
-          const int ib = two ? i2 : 0, jb = two ? j2 : 1;
-          ff ax, ay, az, ae, bx, by, bz, be;
-          pair_term_df(pos[i1], pos[j1], ax, ay, az, ae);
-          pair_term_df(pos[ib], pos[jb], bx, by, bz, be);
-          vb[q] = ax; vb[np + q] = ay; vb[2 * np + q] = az;
-          // cascaded TwoSum (Ogita, Rump and Oishi 2005, Sum2): the high
-          // word's chain is one add; every rounding error and low word goes
-          // to e.lo
-          ff t = ff_two_sum(e.hi, ae.hi);
-          e.hi = t.hi;
-          e.lo = __fadd_rn(e.lo, __fadd_rn(t.lo, ae.lo));
-          if (two) {
-            vb[q + T] = bx; vb[np + q + T] = by; vb[2 * np + q + T] = bz;
-            t = ff_two_sum(e.hi, be.hi);
-            e.hi = t.hi;
-            e.lo = __fadd_rn(e.lo, __fadd_rn(t.lo, be.lo));
-          }
-          pair_advance(n, 2 * T, i1, j1);
-          pair_advance(n, 2 * T, i2, j2);
-        }
+        half_pairs<T>(tm.rank, n, vb,
+                      [&](int i, int j, ff& vx, ff& vy, ff& vz, ff& ep) {
+                        pair_term_df(pos[i], pos[j], vx, vy, vz, ep);
+                      },
+                      [&](ff ep) { df_acc(e_df, ep); });   // reduced below, with g.d
         tm.sync();
-        const float gs = p.k.gs_f;
-        for (int q3 = tm.rank; q3 < 3 * n; q3 += T) {
-          const int ii = q3 / 3;
-          const ff* vc = vb + (q3 - 3 * ii) * np;
-          // All lanes walk j = 0 .. n-1 together (no divergence), four
-          // independent cascaded-TwoSum sums (Sum2, as for the energy),
-          // loads issued a block of four ahead of the adds.
-          const int ri = row_base(n, ii);
-          int rj = -1;                          // row_base(n, j)
-          ff s[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
-          for (int j0 = 0; j0 < n; j0 += 4) {
-            ff v[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              const int j = j0 + u;
-              const int q = j < ii ? rj + ii : ri + j;
-              v[u] = ff{0.f, 0.f};
-              if (j < n && j != ii) v[u] = vc[q];
-              if (j < ii) v[u] = ff{-v[u].hi, -v[u].lo};   // -v over j < i
-              rj += n - j - 2;
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              const ff t = ff_two_sum(s[u].hi, v[u].hi);
-              s[u].hi = t.hi;
-              s[u].lo = __fadd_rn(s[u].lo, __fadd_rn(t.lo, v[u].lo));
-            }
-          }
-          const ff sum = df_add(df_add(s[0], s[1]), df_add(s[2], s[3]));
-          gsum[q3] = -gs * (sum.hi + sum.lo);
-        }
+        half_rows<T>(tm.rank, n, vb, -p.k.gs_f, gsum);
         tm.sync();
-        e_df = e;               // reduced below, together with g.d
       } else {
         const PosD* pos = static_cast<const PosD*>(posv);
         double* vb = static_cast<double*>(hbuf);
         const double sig2 = p.k.sig2;
         dd e{0.0, 0.0};
-        for (int q = tm.rank; q < np; q += 2 * T) {
-          const bool two = q + T < np;
-          const int ib = two ? i2 : 0, jb = two ? j2 : 1;
-          double ax, ay, az, ae, bx, by, bz, be;
-          pair_term_f64(pos[i1], pos[j1], sig2, ax, ay, az, ae);
-          pair_term_f64(pos[ib], pos[jb], sig2, bx, by, bz, be);
-          vb[q] = ax; vb[np + q] = ay; vb[2 * np + q] = az;
-          double eb = ae;
-          if (two) {
-            vb[q + T] = bx; vb[np + q + T] = by; vb[2 * np + q + T] = bz;
-            eb += be;
-          }
-          const dd t = dd_two_sum(e.hi, eb);    // compensated energy sum
-          e.hi = t.hi;
-          e.lo = __dadd_rn(e.lo, t.lo);
-          pair_advance(n, 2 * T, i1, j1);
-          pair_advance(n, 2 * T, i2, j2);
-        }
+        half_pairs<T>(tm.rank, n, vb,
+                      [&](int i, int j, double& vx, double& vy, double& vz, double& ep) {
+                        pair_term_f64(pos[i], pos[j], sig2, vx, vy, vz, ep);
+                      },
+                      [&](double ep) { dd_acc(e, ep); });   // compensated energy sum
         tm.sync();
-        const double gs = p.k.gscale;
-        for (int q3 = tm.rank; q3 < 3 * n; q3 += T) {
-          const int ii = q3 / 3;
-          const double* vc = vb + (q3 - 3 * ii) * np;
-          const int ri = row_base(n, ii);       // same walk as the df sums
-          int rj = -1;
-          double s[4] = {0.0, 0.0, 0.0, 0.0};
-          for (int j0 = 0; j0 < n; j0 += 4) {
-            double v[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              const int j = j0 + u;
-              const int q = j < ii ? rj + ii : ri + j;
-              v[u] = 0.0;
-              if (j < n && j != ii) v[u] = vc[q];
-              if (j < ii) v[u] = -v[u];
-              rj += n - j - 2;
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) s[u] += v[u];
-          }
-          gsum[q3] = -gs * ((s[0] + s[1]) + (s[2] + s[3]));
-        }
+        half_rows<T>(tm.rank, n, vb, -p.k.gscale, gsum);
         tm.sync();
         E = team_sum_dd<T>(tm, e) * p.k.e4;
       }
@@ -638,6 +509,43 @@ __device__ __forceinline__ void evaluate(const Team<T>& tm, int n,
       return;
     }
   }
+  if constexpr ((PM == 1 || std::is_same<X, double>::value) && T * A <= 256) {
+    if (hbuf != nullptr && p.layout == LAYOUT_RING) {
+      if constexpr (PM == 1) {
+        const PosDF* pos = static_cast<const PosDF*>(posv);
+        ff acc[A][3], e{0.f, 0.f};
+        ring_pairs<T, A>(tm, n, p.ring_ks, static_cast<ff*>(hbuf),
+                         [&](int i, int j, ff& vx, ff& vy, ff& vz, ff& ep) {
+                           pair_term_df(pos[i], pos[j], vx, vy, vz, ep);
+                         },
+                         [&](ff ep) { df_acc(e, ep); }, acc);
+        ring_gradient<T, A, P>(tm, n, acc, -p.k.gs_f, g, d, dp);
+        if constexpr (std::is_same<V, float>::value) {
+          if (d) {
+            team_sum_ff_f<T>(tm, e, dp);
+            E = ff_scale(e, p.k.e4_f);
+            dphi = (S)dp;
+            return;
+          }
+        }
+        E = ff_scale(team_sum_ff<T>(tm, e), p.k.e4_f);
+      } else {
+        const PosD* pos = static_cast<const PosD*>(posv);
+        const double sig2 = p.k.sig2;
+        double acc[A][3];
+        dd e{0.0, 0.0};
+        ring_pairs<T, A>(tm, n, p.ring_ks, static_cast<double*>(hbuf),
+                         [&](int i, int j, double& vx, double& vy, double& vz, double& ep) {
+                           pair_term_f64(pos[i], pos[j], sig2, vx, vy, vz, ep);
+                         },
+                         [&](double ep) { dd_acc(e, ep); }, acc);
+        ring_gradient<T, A, P>(tm, n, acc, -p.k.gscale, g, d, dp);
+        E = team_sum_dd<T>(tm, e) * p.k.e4;
+      }
+      if (d) dphi = (S)team_sum1<T, V>(tm, dp);
+      return;
+    }
+  }
   if constexpr (PM == 1) {
     const PosDF* pos = static_cast<const PosDF*>(posv);
     const float gs = p.k.gs_f;
@@ -645,7 +553,7 @@ __device__ __forceinline__ void evaluate(const Team<T>& tm, int n,
     // ---- tiled half-pair evaluation (teams for more than 256 atoms; compiled
     // only for team shapes that can hold them) ------------------------------
     if constexpr (T * A > 256) {
-    if (hbuf != nullptr && p.tiled) {
+    if (hbuf != nullptr && p.layout == LAYOUT_TILES) {
       ff* acc = static_cast<ff*>(hbuf);
       df_tile_eval<T>(tm, n, pos, acc, e);
 #pragma unroll
@@ -728,7 +636,7 @@ __device__ __forceinline__ void evaluate(const Team<T>& tm, int n,
     dd e{0.0, 0.0};
     // ---- tiled FP64 evaluation (teams for more than 256 atoms) -------------
     if constexpr (T * A > 256) {
-    if (hbuf != nullptr && p.tiled) {
+    if (hbuf != nullptr && p.layout == LAYOUT_TILES) {
       double* acc = static_cast<double*>(hbuf);
       d_tile_eval<T>(tm, n, pos, p.k.sig2, acc, e);
 #pragma unroll
@@ -765,16 +673,38 @@ __device__ __forceinline__ void evaluate(const Team<T>& tm, int n,
   if (d) dphi = (S)team_sum1<T, V>(tm, dp);
 }
 
-template <int T, int A, typename X>
-__device__ __forceinline__ X grad_max(const Team<T>& tm, const X (&g)[A][3]) {
-  X m = (X)0;
+// largest |g| of this thread as its bit pattern (NaN: above infinity's): bits of
+// non-negative floats order as integers, so maxima run on the integer pipe
+template <int A>
+__device__ __forceinline__ unsigned max_bits(const float (&g)[A][3]) {
+  unsigned m = 0;
 #pragma unroll
   for (int a = 0; a < A; ++a)
 #pragma unroll
-    for (int c = 0; c < 3; ++c) m = fmax(m, abs_nan_inf(g[a][c]));
-  X v[1] = {m};
-  team_max<T, 1, X>(tm, v);
-  return v[0];
+    for (int c = 0; c < 3; ++c) m = max(m, __float_as_uint(g[a][c]) & 0x7fffffffu);
+  return m;
+}
+template <int A>
+__device__ __forceinline__ unsigned long long max_bits(const double (&g)[A][3]) {
+  unsigned long long m = 0;
+#pragma unroll
+  for (int a = 0; a < A; ++a)
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+      m = max(m, (unsigned long long)__double_as_longlong(g[a][c]) & 0x7fffffffffffffffULL);
+  return m;
+}
+// back to a value; a NaN anywhere gives infinity
+__device__ __forceinline__ float from_bits(unsigned b) {
+  return __uint_as_float(min(b, 0x7f800000u));
+}
+__device__ __forceinline__ double from_bits(unsigned long long b) {
+  return __longlong_as_double((long long)min(b, 0x7ff0000000000000ULL));
+}
+
+template <int T, int A, typename X>
+__device__ __forceinline__ X grad_max(const Team<T>& tm, const X (&g)[A][3]) {
+  return from_bits(team_max_bits(tm, max_bits(g)));
 }
 
 // Sufficient decrease f(a) <= f(0) + c1 a phi'(0).  FP64-valued energies use
@@ -850,196 +780,247 @@ __device__ __forceinline__ void warp_sum2(V& v0, V& v1) {
   }
 }
 
+// The vectors lie flat (3 N values, zeros behind them): lane l holds 16 bytes
+// of every 512, one vector load and at most four values a lane for LJ38 where
+// a lane with the atoms l and l + 32 had six, and while a block's products are
+// being reduced its other vectors and the next block's are on their way.  1/s.y, s.y/y.y,
+// s_{t-1}.y_t and alpha are a register each, slot t's in lane t.
+// In isolation (one team, m = 10, N = 38) a direction takes 3.5k cycles: ~290 a
+// block of two pairs, 175 of them the two-value reduction, and ~570 once.
+// LJ38 Basin Hopping near its minima (64 walkers x 8, 25 steps, mixed): 11.8 ms a
+// launch before this form, one evaluation in the line search (run_phase) and the
+// ring order of the half pairs, 9.9 after.
+// ---------------------------------------------------------------------------
+// 16 bytes of a vector: its part of a dot product and of an update.  FP32
+// takes two values an instruction.
+template <typename V>
+struct HistVec;
+template <>
+struct HistVec<float> {
+  static constexpr int W = 4;
+  float2 a, b;
+  __device__ __forceinline__ void load(const float* p) {
+    const float4 q = *reinterpret_cast<const float4*>(p);
+    a = make_float2(q.x, q.y);
+    b = make_float2(q.z, q.w);
+  }
+  __device__ __forceinline__ void store(float* p) const {
+    *reinterpret_cast<float4*>(p) = make_float4(a.x, a.y, b.x, b.y);
+  }
+  __device__ __forceinline__ void zero() { a = f2(0.f); b = f2(0.f); }
+  __device__ __forceinline__ void scale(float c) { a = __fmul2_rn(a, f2(c)); b = __fmul2_rn(b, f2(c)); }
+  __device__ __forceinline__ void add(float c, const HistVec& o) {
+    a = __ffma2_rn(f2(c), o.a, a);
+    b = __ffma2_rn(f2(c), o.b, b);
+  }
+};
+template <>
+struct HistVec<double> {
+  static constexpr int W = 2;
+  double a, b;
+  __device__ __forceinline__ void load(const double* p) {
+    const double2 q = *reinterpret_cast<const double2*>(p);
+    a = q.x;
+    b = q.y;
+  }
+  __device__ __forceinline__ void store(double* p) const {
+    *reinterpret_cast<double2*>(p) = make_double2(a, b);
+  }
+  __device__ __forceinline__ void zero() { a = 0.0; b = 0.0; }
+  __device__ __forceinline__ void scale(double c) { a *= c; b *= c; }
+  __device__ __forceinline__ void add(double c, const HistVec& o) {
+    a = fma(c, o.a, a);
+    b = fma(c, o.b, b);
+  }
+};
+template <int NC>
+__device__ __forceinline__ float hist_dot(const HistVec<float> (&x)[NC], const HistVec<float> (&y)[NC]) {
+  float2 s = __fmul2_rn(x[0].a, y[0].a);
+  s = __ffma2_rn(x[0].b, y[0].b, s);
+#pragma unroll
+  for (int c = 1; c < NC; ++c) {
+    s = __ffma2_rn(x[c].a, y[c].a, s);
+    s = __ffma2_rn(x[c].b, y[c].b, s);
+  }
+  return __fadd_rn(s.x, s.y);
+}
+template <int NC>
+__device__ __forceinline__ double hist_dot(const HistVec<double> (&x)[NC],
+                                           const HistVec<double> (&y)[NC]) {
+  double s = x[0].a * y[0].a;
+  s = fma(x[0].b, y[0].b, s);
+#pragma unroll
+  for (int c = 1; c < NC; ++c) {
+    s = fma(x[c].a, y[c].a, s);
+    s = fma(x[c].b, y[c].b, s);
+  }
+  return s;
+}
+
+// 1 / s.y, s.y / y.y and s_prev.y of the stored pairs.  LANES: slot t's in
+// lane t of every warp, read by a shuffle (teams whose first warp runs the
+// recursion); else in an array of every thread.
+template <typename V, bool LANES>
+struct PairScalars {
+  V rho = (V)0, gam = (V)0, sup = (V)0;
+  __device__ __forceinline__ V rho_of(int sl) const { return __shfl_sync(kFull, rho, sl); }
+  __device__ __forceinline__ V gam_of(int sl) const { return __shfl_sync(kFull, gam, sl); }
+  __device__ __forceinline__ V sup_of(int sl) const { return __shfl_sync(kFull, sup, sl); }
+  __device__ __forceinline__ void set(int rank, int sl, V r, V g, V u) {
+    if ((rank & 31) == sl) { rho = r; gam = g; sup = u; }
+  }
+};
+template <typename V>
+struct PairScalars<V, false> {
+  V rho[LJ_MAX_M], gam[LJ_MAX_M];
+  __device__ __forceinline__ V rho_of(int sl) const { return rho[sl]; }
+  __device__ __forceinline__ V gam_of(int sl) const { return gam[sl]; }
+  __device__ __forceinline__ void set(int, int sl, V r, V g, V) { rho[sl] = r; gam[sl] = g; }
+};
+
+// the recursion of the lead warp on vectors of NC chunks of 512 bytes: q (the
+// gradient, in xb) to the direction (in xb), returns g.d
+template <int L3, int NC, typename V>
+__device__ __forceinline__ V lead_recursion(int lane, int m, int cnt, int head,
+                                            const V* __restrict__ Sh, const V* __restrict__ Yh,
+                                            const PairScalars<V, true>& ps, V* xb) {
+  using Vec = HistVec<V>;
+  constexpr int W = Vec::W;
+  Vec q[NC], d0[NC], d1[NC], u0[NC], u1[NC];
+  auto load = [&](const V* base, Vec (&o)[NC]) {
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      const int f = (c * 32 + lane) * W;
+      if ((c + 1) * 32 * W <= L3) {          // whole chunks
+        o[c].load(base + f);
+      } else {
+        o[c].zero();
+        if (f < L3) o[c].load(base + f);
+      }
+    }
+  };
+  // slots of the pairs t (newest: cnt - 1); where there is no such pair, the
+  // nearest one, whose factor is then zero: a branch around a shuffle or a
+  // load, whose condition the compiler cannot know to be uniform, costs more
+  // than reading a pair too many
+  auto older = [&](int k, bool is) { return !is ? k : k == 0 ? m - 1 : k - 1; };
+  auto newer = [&](int k, bool is) { return !is ? k : k == m - 1 ? 0 : k + 1; };
+  load(xb, q);
+  V alpha = (V)0;
+  // ---- first loop, newest first ----------------------------------------------
+  int k0 = head + cnt - 1;
+  if (k0 >= m) k0 -= m;
+  const V gam = ps.gam_of(k0);
+  int k1 = older(k0, cnt >= 2);
+  constexpr bool kAhead = NC <= 3;           // registers for the next block's vectors
+  if (kAhead) {
+    load(Sh + k0 * L3, d0);
+    load(Sh + k1 * L3, d1);
+  }
+  for (int t = cnt - 1; t >= 0; t -= 2) {
+    if (!kAhead) {
+      load(Sh + k0 * L3, d0);
+      load(Sh + k1 * L3, d1);
+    }
+    V p0 = hist_dot(d0, q), p1 = hist_dot(d1, q);
+    // in flight during the reduction: this block's y, the next block's s
+    load(Yh + k0 * L3, u0);
+    load(Yh + k1 * L3, u1);
+    const V r0 = ps.rho_of(k0), u = ps.sup_of(k0);
+    V r1 = ps.rho_of(k1);
+    if (t < 1) r1 = (V)0;
+    k0 = older(k1, t >= 2);
+    k1 = older(k0, t >= 3);
+    if (kAhead) {
+      load(Sh + k0 * L3, d0);
+      load(Sh + k1 * L3, d1);
+    }
+    warp_sum2(p0, p1);
+    const V a0 = r0 * p0;
+    const V a1 = r1 * (p1 - a0 * u);
+    if (lane == t) alpha = a0;
+    if (lane == t - 1) alpha = a1;
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      q[c].add(-a0, u0[c]);
+      q[c].add(-a1, u1[c]);
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < NC; ++c) q[c].scale(gam);
+  // ---- second loop, oldest first ----------------------------------------------
+  k0 = head;
+  k1 = newer(k0, cnt >= 2);
+  if (kAhead) {
+    load(Yh + k0 * L3, d0);
+    load(Yh + k1 * L3, d1);
+  }
+  for (int t = 0; t < cnt; t += 2) {
+    if (!kAhead) {
+      load(Yh + k0 * L3, d0);
+      load(Yh + k1 * L3, d1);
+    }
+    V p0 = hist_dot(d0, q), p1 = hist_dot(d1, q);
+    load(Sh + k0 * L3, u0);
+    load(Sh + k1 * L3, u1);
+    const V r0 = ps.rho_of(k0), r1 = ps.rho_of(k1), u = ps.sup_of(k1);
+    const V al0 = __shfl_sync(kFull, alpha, t), al1 = __shfl_sync(kFull, alpha, (t + 1) & 31);
+    k0 = newer(k1, t + 2 < cnt);
+    k1 = newer(k0, t + 3 < cnt);
+    if (kAhead) {
+      load(Yh + k0 * L3, d0);
+      load(Yh + k1 * L3, d1);
+    }
+    warp_sum2(p0, p1);
+    const V c0 = al0 - r0 * p0;
+    V c1 = al1 - r1 * (p1 + c0 * u);
+    if (t + 1 >= cnt) c1 = (V)0;
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      q[c].add(c0, u0[c]);
+      q[c].add(c1, u1[c]);
+    }
+  }
+  load(xb, d0);
+  const V dphi = -warp_sum(hist_dot(d0, q));
+#pragma unroll
+  for (int c = 0; c < NC; ++c) {
+    const int f = (c * 32 + lane) * W;
+    q[c].scale((V)-1);
+    if ((c + 1) * 32 * W <= L3 || f < L3) q[c].store(xb + f);
+  }
+  return dphi;
+}
+
 template <int T, int A, typename XG, typename V>
-__device__ __forceinline__ V lead_two_loop(const Team<T>& tm, int m, int cnt, int head,
+__device__ __forceinline__ V lead_two_loop(const Team<T>& tm, int n, int m, int cnt, int head,
                                            const V* __restrict__ Sh, const V* __restrict__ Yh,
-                                           const V (&rho)[LJ_MAX_M], const V (&gmv)[LJ_MAX_M],
-                                           const V (&sup)[LJ_MAX_M], const XG (&g)[A][3],
+                                           const PairScalars<V, true>& ps, const XG (&g)[A][3],
                                            V* xb, V (&d)[A][3]) {
-  constexpr int W = T / 32;
+  constexpr int L3 = 3 * A * T;               // values of a slot
+  constexpr int CH = 32 * HistVec<V>::W;
+  constexpr int NC = (L3 + CH - 1) / CH;
 #pragma unroll
   for (int a = 0; a < A; ++a)
 #pragma unroll
-    for (int c = 0; c < 3; ++c) xb[(a * 3 + c) * T + tm.rank] = (V)g[a][c];
+    for (int c = 0; c < 3; ++c) xb[3 * (a * T + tm.rank) + c] = (V)g[a][c];
   tm.sync();
   if (tm.rank < 32) {
-    const int lane = tm.rank;
-    auto slot_of = [&](int t) { const int sl = head + t; return sl >= m ? sl - m : sl; };
-    V q[W][A][3], gl[W][A][3];
-    V alpha[LJ_MAX_M];
-#pragma unroll
-    for (int w = 0; w < W; ++w)
-#pragma unroll
-      for (int a = 0; a < A; ++a)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          gl[w][a][c] = xb[(a * 3 + c) * T + lane + 32 * w];
-          q[w][a][c] = gl[w][a][c];
-        }
-    // ---- first loop, newest first --------------------------------------------
-    int t = cnt - 1;
-    for (; t >= 1; t -= 2) {
-      const int s0 = slot_of(t), s1 = slot_of(t - 1);
-      V sv0[W][A][3], yv0[W][A][3], sv1[W][A][3], yv1[W][A][3];
-#pragma unroll
-      for (int w = 0; w < W; ++w)
-#pragma unroll
-        for (int a = 0; a < A; ++a)
-#pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            sv0[w][a][c] = Sh[hidx<T, A>(s0, a, c, lane + 32 * w)];
-            yv0[w][a][c] = Yh[hidx<T, A>(s0, a, c, lane + 32 * w)];
-            sv1[w][a][c] = Sh[hidx<T, A>(s1, a, c, lane + 32 * w)];
-            yv1[w][a][c] = Yh[hidx<T, A>(s1, a, c, lane + 32 * w)];
-          }
-      const V r0 = rho[s0], r1 = rho[s1], u01 = sup[s0];
-      V p0 = (V)0, p1 = (V)0;
-#pragma unroll
-      for (int w = 0; w < W; ++w)
-#pragma unroll
-        for (int a = 0; a < A; ++a)
-#pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            p0 += sv0[w][a][c] * q[w][a][c];
-            p1 += sv1[w][a][c] * q[w][a][c];
-          }
-      warp_sum2(p0, p1);
-      const V a0 = r0 * p0;
-      const V a1 = r1 * (p1 - a0 * u01);
-      alpha[t] = a0;
-      alpha[t - 1] = a1;
-#pragma unroll
-      for (int w = 0; w < W; ++w)
-#pragma unroll
-        for (int a = 0; a < A; ++a)
-#pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            q[w][a][c] -= a0 * yv0[w][a][c];
-            q[w][a][c] -= a1 * yv1[w][a][c];
-          }
-    }
-    if (t == 0) {
-      const int s0 = slot_of(0);
-      V sv0[W][A][3], yv0[W][A][3];
-#pragma unroll
-      for (int w = 0; w < W; ++w)
-#pragma unroll
-        for (int a = 0; a < A; ++a)
-#pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            sv0[w][a][c] = Sh[hidx<T, A>(s0, a, c, lane + 32 * w)];
-            yv0[w][a][c] = Yh[hidx<T, A>(s0, a, c, lane + 32 * w)];
-          }
-      V part = (V)0;
-#pragma unroll
-      for (int w = 0; w < W; ++w)
-#pragma unroll
-        for (int a = 0; a < A; ++a)
-#pragma unroll
-          for (int c = 0; c < 3; ++c) part += sv0[w][a][c] * q[w][a][c];
-      const V a0 = rho[s0] * warp_sum(part);
-      alpha[0] = a0;
-#pragma unroll
-      for (int w = 0; w < W; ++w)
-#pragma unroll
-        for (int a = 0; a < A; ++a)
-#pragma unroll
-          for (int c = 0; c < 3; ++c) q[w][a][c] -= a0 * yv0[w][a][c];
-    }
-    const V gam = gmv[slot_of(cnt - 1)];
-#pragma unroll
-    for (int w = 0; w < W; ++w)
-#pragma unroll
-      for (int a = 0; a < A; ++a)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) q[w][a][c] *= gam;
-    // ---- second loop, oldest first ---------------------------------------------
-    t = 0;
-    for (; t + 1 < cnt; t += 2) {
-      const int s0 = slot_of(t), s1 = slot_of(t + 1);
-      V sv0[W][A][3], yv0[W][A][3], sv1[W][A][3], yv1[W][A][3];
-#pragma unroll
-      for (int w = 0; w < W; ++w)
-#pragma unroll
-        for (int a = 0; a < A; ++a)
-#pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            sv0[w][a][c] = Sh[hidx<T, A>(s0, a, c, lane + 32 * w)];
-            yv0[w][a][c] = Yh[hidx<T, A>(s0, a, c, lane + 32 * w)];
-            sv1[w][a][c] = Sh[hidx<T, A>(s1, a, c, lane + 32 * w)];
-            yv1[w][a][c] = Yh[hidx<T, A>(s1, a, c, lane + 32 * w)];
-          }
-      const V r0 = rho[s0], r1 = rho[s1], u01 = sup[s1];
-      const V al0 = alpha[t], al1 = alpha[t + 1];
-      V p0 = (V)0, p1 = (V)0;
-#pragma unroll
-      for (int w = 0; w < W; ++w)
-#pragma unroll
-        for (int a = 0; a < A; ++a)
-#pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            p0 += yv0[w][a][c] * q[w][a][c];
-            p1 += yv1[w][a][c] * q[w][a][c];
-          }
-      warp_sum2(p0, p1);
-      const V c0 = al0 - r0 * p0;
-      const V c1 = al1 - r1 * (p1 + c0 * u01);
-#pragma unroll
-      for (int w = 0; w < W; ++w)
-#pragma unroll
-        for (int a = 0; a < A; ++a)
-#pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            q[w][a][c] += c0 * sv0[w][a][c];
-            q[w][a][c] += c1 * sv1[w][a][c];
-          }
-    }
-    if (t < cnt) {
-      const int s0 = slot_of(t);
-      V sv0[W][A][3], yv0[W][A][3];
-#pragma unroll
-      for (int w = 0; w < W; ++w)
-#pragma unroll
-        for (int a = 0; a < A; ++a)
-#pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            sv0[w][a][c] = Sh[hidx<T, A>(s0, a, c, lane + 32 * w)];
-            yv0[w][a][c] = Yh[hidx<T, A>(s0, a, c, lane + 32 * w)];
-          }
-      V part = (V)0;
-#pragma unroll
-      for (int w = 0; w < W; ++w)
-#pragma unroll
-        for (int a = 0; a < A; ++a)
-#pragma unroll
-          for (int c = 0; c < 3; ++c) part += yv0[w][a][c] * q[w][a][c];
-      const V c0 = alpha[t] - rho[s0] * warp_sum(part);
-#pragma unroll
-      for (int w = 0; w < W; ++w)
-#pragma unroll
-        for (int a = 0; a < A; ++a)
-#pragma unroll
-          for (int c = 0; c < 3; ++c) q[w][a][c] += c0 * sv0[w][a][c];
-    }
-    V part = (V)0;
-#pragma unroll
-    for (int w = 0; w < W; ++w)
-#pragma unroll
-      for (int a = 0; a < A; ++a)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          xb[(a * 3 + c) * T + lane + 32 * w] = -q[w][a][c];
-          part += gl[w][a][c] * -q[w][a][c];
-        }
-    const V dphi = warp_sum(part);
-    if (lane == 0) xb[A * 3 * T] = dphi;
+    // clusters that leave the last third or more of the chunks empty: fewer
+    constexpr int ND = NC > 2 ? NC * 2 / 3 : 1;
+    const V dphi = NC > 1 && 3 * n <= ND * CH
+                       ? lead_recursion<L3, ND, V>(tm.rank, m, cnt, head, Sh, Yh, ps, xb)
+                       : lead_recursion<L3, NC, V>(tm.rank, m, cnt, head, Sh, Yh, ps, xb);
+    if (NC > 1 && 3 * n <= ND * CH)           // zeros behind the chunks that were taken
+      for (int f = ND * CH + tm.rank; f < L3; f += 32) xb[f] = (V)0;
+    if (tm.rank == 0) xb[L3] = dphi;
   }
   tm.sync();
 #pragma unroll
   for (int a = 0; a < A; ++a)
 #pragma unroll
-    for (int c = 0; c < 3; ++c) d[a][c] = xb[(a * 3 + c) * T + tm.rank];
-  return xb[A * 3 * T];
+    for (int c = 0; c < 3; ++c) d[a][c] = xb[3 * (a * T + tm.rank) + c];
+  return xb[L3];
 }
 
 // ---------------------------------------------------------------------------
@@ -1064,9 +1045,7 @@ template <int T, int A, typename P, int MODE>
 __device__ __forceinline__ int run_phase(const Team<T>& tm, int n, typename P::XP (&x)[A][3],
                          typename P::XG (&g)[A][3], typename P::F& f,
                          typename P::V* __restrict__ Sh, typename P::V* __restrict__ Yh,
-                         typename P::V (&rho)[LJ_MAX_M], typename P::V (&gmv)[LJ_MAX_M],
-                         typename P::V (&sup)[LJ_MAX_M], int& cnt,
-                         int& head, int& iters,
+                         PairScalars<typename P::V, (T <= 128)>& ps, int& cnt, int& head, int& iters,
                          int& evals, int& phase_iters, long long& vec, void* pos,
                          void* hbuf, const MinParams& p, long long t0, long long (&cyc)[2]) {
   using X = typename P::XP;
@@ -1078,7 +1057,6 @@ __device__ __forceinline__ int run_phase(const Team<T>& tm, int n, typename P::X
   const S c1 = (S)p.c1, c2 = (S)p.c2, amax = (S)p.alpha_max;
   const S resolution = (S)(MODE == 1 ? p.f32_resolution : p.df_resolution);
   const XG stop_gtol = MODE == 1 ? (XG)p.switch_gtol : (XG)p.gtol;
-  V alpha[LJ_MAX_M];
   V d[A][3];
   bool gmode = false;   // MODE 1, 2: energy below resolution, gradient-only line search
   X xt[A][3];
@@ -1096,11 +1074,12 @@ __device__ __forceinline__ int run_phase(const Team<T>& tm, int n, typename P::X
       if constexpr (std::is_same<V, float>::value) {
         if (12 * A * T + 4 <= 32 * n) xb = static_cast<V*>(pos);
       } else {
-        if (hbuf != nullptr && !p.tiled && 24 * A * T + 8 <= 24 * n_pairs(n))
+        if (hbuf != nullptr && (p.layout == LAYOUT_RING ||
+                                (p.layout == LAYOUT_HALF && 24 * A * T + 8 <= 24 * n_pairs(n))))
           xb = static_cast<V*>(hbuf);
       }
       if (cnt > 0 && xb != nullptr) {
-        dphi0 = (S)lead_two_loop<T, A, XG, V>(tm, m, cnt, head, Sh, Yh, rho, gmv, sup, g, xb, d);
+        dphi0 = (S)lead_two_loop<T, A, XG, V>(tm, n, m, cnt, head, Sh, Yh, ps, g, xb, d);
         vec += (long long)cnt * 3 * n;
         led = true;
       }
@@ -1114,6 +1093,7 @@ __device__ __forceinline__ int run_phase(const Team<T>& tm, int n, typename P::X
       // two-loop recursion; each step prefetches the next pair's vectors and
       // 1/s.y before its own team reduction, so loads overlap the reduction
       auto slot_of = [&](int t) { const int sl = head + t; return sl >= m ? sl - m : sl; };
+      V alpha[LJ_MAX_M];
       V sc[A][3], yc[A][3], sn[A][3], yn[A][3];
       {
         const int sl = slot_of(cnt - 1);
@@ -1125,7 +1105,7 @@ __device__ __forceinline__ int run_phase(const Team<T>& tm, int n, typename P::X
             yc[a][c] = Yh[hidx<T, A>(sl, a, c, tm.rank)];
           }
       }
-      V rho_c = rho[slot_of(cnt - 1)];
+      V rho_c = ps.rho_of(slot_of(cnt - 1));
       for (int t = cnt - 1; t >= 0; --t) {
         const int nsl = slot_of(t > 0 ? t - 1 : 0);
 #pragma unroll
@@ -1135,7 +1115,7 @@ __device__ __forceinline__ int run_phase(const Team<T>& tm, int n, typename P::X
             sn[a][c] = Sh[hidx<T, A>(nsl, a, c, tm.rank)];
             yn[a][c] = Yh[hidx<T, A>(nsl, a, c, tm.rank)];
           }
-        const V rho_n = rho[nsl];
+        const V rho_n = ps.rho_of(nsl);
         V part = (V)0;
 #pragma unroll
         for (int a = 0; a < A; ++a)
@@ -1154,13 +1134,13 @@ __device__ __forceinline__ int run_phase(const Team<T>& tm, int n, typename P::X
         rho_c = rho_n;
       }
       const int newest = slot_of(cnt - 1);
-      const V gam = gmv[newest];
+      const V gam = ps.gam_of(newest);
 #pragma unroll
       for (int a = 0; a < A; ++a)
 #pragma unroll
         for (int c = 0; c < 3; ++c) q[a][c] *= gam;
       // (sc, yc) now hold the oldest pair, the first one of the second loop
-      rho_c = rho[slot_of(0)];
+      rho_c = ps.rho_of(slot_of(0));
       for (int t = 0; t < cnt; ++t) {
         const int nsl = slot_of(t + 1 < cnt ? t + 1 : t);
 #pragma unroll
@@ -1170,7 +1150,7 @@ __device__ __forceinline__ int run_phase(const Team<T>& tm, int n, typename P::X
             sn[a][c] = Sh[hidx<T, A>(nsl, a, c, tm.rank)];
             yn[a][c] = Yh[hidx<T, A>(nsl, a, c, tm.rank)];
           }
-        const V rho_n = rho[nsl];
+        const V rho_n = ps.rho_of(nsl);
         V part = (V)0;
 #pragma unroll
         for (int a = 0; a < A; ++a)
@@ -1244,8 +1224,13 @@ __device__ __forceinline__ int run_phase(const Team<T>& tm, int n, typename P::X
         // is trusted down to switch_gtol, the double-float one to ~1e-11)
         if (-dphi0 * a1 < resolution * fabsf(f.hi)) gmode = true;
       }
-      // ---- strong-Wolfe line search ----------------------------------------
-      int ev = 0;
+      // ---- line search --------------------------------------------------------
+      // One loop with one evaluation in it: its four kinds of trial (bracketing
+      // and zoom of the strong-Wolfe search, the gradient-only search, and the
+      // best point once more when the budget is spent) share the code of the
+      // evaluation, which inlined at each of them filled the instruction cache.
+      enum { BRACKET, ZOOM, GRAD, LAST };
+      int kind = BRACKET, ev = 0;
       S a_prev = (S)0, dp_prev = dphi0;
       F f_prev = f;
       S a = a1;
@@ -1254,112 +1239,113 @@ __device__ __forceinline__ int run_phase(const Team<T>& tm, int n, typename P::X
       F best_f = f;
       S lo = 0, hi = 0, dp_lo = 0, dp_hi = 0;
       F f_lo = f, f_hi = f;
-      S dp;
-      bool done = false, zoom = false;
-      auto trial = [&](S al, F& fo, S& dpo) {
+      bool done = false;
+      // gradient-only search (approximate Wolfe conditions, Hager and Zhang
+      // 2005): accept |phi'(a)| <= c2 |phi'(0)| with the energy no more than
+      // the resolution above f(0) (which, for a near-quadratic phi, also
+      // implies the Armijo decrease); bracket on the sign of phi' and
+      // interpolate by secant steps on phi'.  lo, dp_lo: the last point too
+      // short; hi, dp_hi: the first too long (hi < 0: none)
+      S tol_f = (S)0;
+      bool hi_slope = false;
+      if constexpr (MODE == 1 || MODE == 2) {
+        if (gmode) {
+          kind = GRAD;
+          tol_f = (S)2 * resolution * fabsf(f.hi);
+          hi = (S)-1;
+          dp_lo = dphi0;
+        }
+      }
+      for (int i = 1;; ++i) {
+        if (ev >= p.max_ls) {
+          // out of budget: the best point with sufficient decrease, if it is lower
+          if (kind == GRAD || !have_best || !((S)fdiff(best_f, f) < (S)0)) break;
+          if (last_a == best_a) {
+            ft = best_f;
+            done = true;
+            break;
+          }
+          kind = LAST;
+          a = best_a;
+        }
+        F fa;
+        S dp;
 #pragma unroll
         for (int aa = 0; aa < A; ++aa)
 #pragma unroll
-          for (int c = 0; c < 3; ++c) xt[aa][c] = pos_step(x[aa][c], al, d[aa][c]);
-        evaluate<T, A, P>(tm, n, xt, gt, pos, hbuf, p, d, fo, dpo);
+          for (int c = 0; c < 3; ++c) xt[aa][c] = pos_step(x[aa][c], a, d[aa][c]);
+        evaluate<T, A, P>(tm, n, xt, gt, pos, hbuf, p, d, fa, dp);
         ++ev;
-        last_a = al;
-      };
-      bool gsearch = false;
-      if constexpr (MODE == 1 || MODE == 2) {
-      if (gmode) {
-        gsearch = true;
-        // ---- gradient-only search (approximate Wolfe conditions, Hager and
-        // Zhang 2005): accept |phi'(a)| <= c2 |phi'(0)| with the energy no
-        // more than the resolution above f(0) (which, for a near-quadratic
-        // phi, also implies the Armijo decrease); bracket on the sign of
-        // phi' and interpolate by secant steps on phi'.
-        const S tol_f = (S)2 * resolution * fabsf(f.hi);
-        S glo = (S)0, ghi = (S)-1, dlo = dphi0, dhi = (S)0;
-        bool hi_slope = false;
-        while (ev < p.max_ls) {
-          F fa;
-          trial(a, fa, dp);
-          const bool eok = fisfinite(fa) && isfinite(dp) && (S)fdiff(fa, f) <= tol_f;
-          if (!eok || dp > -c2 * dphi0) {          // too long
-            ghi = a; dhi = dp; hi_slope = eok;
-          } else if (dp < c2 * dphi0) {            // too short
-            glo = a; dlo = dp;
-          } else {
-            ft = fa; done = true;
-            break;
-          }
-          if (ghi < (S)0) {
-            a = (S)2 * a;
-            if (a > amax) a = amax;
-          } else {
-            const S w = ghi - glo;
-            S t = (hi_slope && dhi > dlo) ? glo - dlo * w / (dhi - dlo) : glo + (S)0.5 * w;
-            const S tlo = glo + (S)0.1 * w, thi = ghi - (S)0.1 * w;
-            if (!(t >= tlo)) t = tlo;
-            if (!(t <= thi)) t = thi;
-            a = t;
+        last_a = a;
+        if (kind == LAST) {
+          ft = fa;
+          done = true;
+          break;
+        }
+        if constexpr (MODE == 1 || MODE == 2) {
+          if (kind == GRAD) {
+            const bool eok = fisfinite(fa) && isfinite(dp) && (S)fdiff(fa, f) <= tol_f;
+            if (!eok || dp > -c2 * dphi0) {          // too long
+              hi = a; dp_hi = dp; hi_slope = eok;
+            } else if (dp < c2 * dphi0) {            // too short
+              lo = a; dp_lo = dp;
+            } else {
+              ft = fa;
+              done = true;
+              break;
+            }
+            if (hi < (S)0) {
+              a = (S)2 * a;
+              if (a > amax) a = amax;
+            } else {
+              const S w = hi - lo;
+              S t = (hi_slope && dp_hi > dp_lo) ? lo - dp_lo * w / (dp_hi - dp_lo)
+                                                : lo + (S)0.5 * w;
+              const S tlo = lo + (S)0.1 * w, thi = hi - (S)0.1 * w;
+              if (!(t >= tlo)) t = tlo;
+              if (!(t <= thi)) t = thi;
+              a = t;
+            }
+            continue;
           }
         }
-      }
-      }
-      if (!gsearch) {
-      for (int i = 1; !done && !zoom; ++i) {
-        if (ev >= p.max_ls) break;
-        F fa;
-        trial(a, fa, dp);
         const bool armijo = armijo_ok(fa, f, c1 * a * dphi0);
         if (armijo && (!have_best || (S)fdiff(fa, best_f) < (S)0)) {
           have_best = true; best_f = fa; best_a = a;
         }
-        if (!armijo || (i > 1 && (S)fdiff(fa, f_prev) >= (S)0)) {
-          lo = a_prev; f_lo = f_prev; dp_lo = dp_prev;
+        if (kind == BRACKET) {
+          if (!armijo || (i > 1 && (S)fdiff(fa, f_prev) >= (S)0)) {
+            lo = a_prev; f_lo = f_prev; dp_lo = dp_prev;
+            hi = a; f_hi = fa; dp_hi = dp;
+            kind = ZOOM;
+          } else if (fabs(dp) <= -c2 * dphi0) {
+            ft = fa;
+            done = true;
+            break;
+          } else if (dp >= (S)0) {
+            lo = a; f_lo = fa; dp_lo = dp;
+            hi = a_prev; f_hi = f_prev; dp_hi = dp_prev;
+            kind = ZOOM;
+          } else {
+            a_prev = a; f_prev = fa; dp_prev = dp;
+            a = (S)2 * a;
+            if (a > amax) a = amax;
+            continue;
+          }
+        } else if (!armijo || (S)fdiff(fa, f_lo) >= (S)0) {
           hi = a; f_hi = fa; dp_hi = dp;
-          zoom = true;
-        } else if (fabs(dp) <= -c2 * dphi0) {
-          ft = fa; done = true;
-        } else if (dp >= (S)0) {
-          lo = a; f_lo = fa; dp_lo = dp;
-          hi = a_prev; f_hi = f_prev; dp_hi = dp_prev;
-          zoom = true;
-        } else {
-          a_prev = a; f_prev = fa; dp_prev = dp;
-          a = (S)2 * a;
-          if (a > amax) a = amax;
-        }
-      }
-      while (zoom && !done) {
-        if (ev >= p.max_ls) break;
-        const S aj = cubic_step<S, F>(lo, f_lo, dp_lo, hi, f_hi, dp_hi);
-        F fa;
-        trial(aj, fa, dp);
-        const bool armijo = armijo_ok(fa, f, c1 * aj * dphi0);
-        if (armijo && (!have_best || (S)fdiff(fa, best_f) < (S)0)) {
-          have_best = true; best_f = fa; best_a = aj;
-        }
-        if (!armijo || (S)fdiff(fa, f_lo) >= (S)0) {
-          hi = aj; f_hi = fa; dp_hi = dp;
         } else {
           if (fabs(dp) <= -c2 * dphi0) {
-            ft = fa; done = true;
-          } else {
-            if (dp * (hi - lo) >= (S)0) {
-              hi = lo; f_hi = f_lo; dp_hi = dp_lo;
-            }
-            lo = aj; f_lo = fa; dp_lo = dp;
+            ft = fa;
+            done = true;
+            break;
           }
+          if (dp * (hi - lo) >= (S)0) {
+            hi = lo; f_hi = f_lo; dp_hi = dp_lo;
+          }
+          lo = a; f_lo = fa; dp_lo = dp;
         }
-      }
-      if (!done && have_best && (S)fdiff(best_f, f) < (S)0) {
-        if (last_a != best_a) {
-          F fa;
-          trial(best_a, fa, dp);
-          ft = fa;
-        } else {
-          ft = best_f;
-        }
-        done = true;
-      }
+        a = cubic_step<S, F>(lo, f_lo, dp_lo, hi, f_hi, dp_hi);
       }
       evals += ev;
       ok = done;
@@ -1385,14 +1371,9 @@ __device__ __forceinline__ int run_phase(const Team<T>& tm, int n, typename P::X
       }
     // stopping-test values of the new point (||g||_inf, deadline), reduced
     // in the same pass as the curvature pair's s.y and y.y
-    XG mv[2];
-    mv[0] = (XG)0;
-#pragma unroll
-    for (int a = 0; a < A; ++a)
-#pragma unroll
-      for (int c = 0; c < 3; ++c) mv[0] = fmax(mv[0], abs_nan_inf(gt[a][c]));
-    mv[1] = (p.deadline > 0 && (clock64() - t0) > p.deadline) ? (XG)1 : (XG)0;
-    team_sums_max2<T, V, XG>(tm, pr, mv);
+    auto gmax = max_bits(gt);
+    bool late = p.deadline > 0 && (clock64() - t0) > p.deadline;
+    team_sums_max(tm, pr, gmax, late);
     if (pr[0] > eps_mach<V>() * pr[1]) {
       int slot;
       if (cnt < m) {
@@ -1410,9 +1391,9 @@ __device__ __forceinline__ int run_phase(const Team<T>& tm, int n, typename P::X
           Sh[hidx<T, A>(slot, a, c, tm.rank)] = sv[a][c];
           Yh[hidx<T, A>(slot, a, c, tm.rank)] = yv[a][c];
         }
-      rho[slot] = (V)1 / pr[0];      // rho = 1 / s.y and the scaling s.y / y.y, formed
-      gmv[slot] = pr[0] / pr[1];     // once here instead of in every recursion step
-      sup[slot] = pr[2];             // s_prev . y (undefined for the oldest pair: unused)
+      // 1 / s.y and the scaling s.y / y.y, formed once here instead of in every
+      // recursion step; s_prev . y (undefined for the oldest pair: unused)
+      ps.set(tm.rank, slot, recip(pr[0]), pr[0] * recip(pr[1]), pr[2]);
     }
 #pragma unroll
     for (int a = 0; a < A; ++a)
@@ -1425,8 +1406,8 @@ __device__ __forceinline__ int run_phase(const Team<T>& tm, int n, typename P::X
     ++iters;
     ++phase_iters;
     // ---- stopping tests (values reduced above) -----------------------------
-    if (mv[0] < stop_gtol) return MODE == 1 ? PH_SWITCH : PH_CONVERGED;
-    if (mv[1] > (XG)0) return PH_TIMEOUT;
+    if (from_bits(gmax) < stop_gtol) return MODE == 1 ? PH_SWITCH : PH_CONVERGED;
+    if (late) return PH_TIMEOUT;
     if constexpr (MODE == 1) {
       // a switch_gtol below the FP32 gradient noise would keep gradient-only
       // FP32 steps iterating on noise: past kFP32GradIters iterations of the
@@ -1487,9 +1468,9 @@ __device__ __forceinline__ void minimise(const Team<T>& tm, int n, double (&x64)
       r.E = f; r.status = ST_NONFINITE; lap(r.cyc64); return;
     }
     if (gm < p.gtol) { r.E = f; lap(r.cyc64); return; }
-    double rho[LJ_MAX_M], gmv[LJ_MAX_M], sup[LJ_MAX_M];
+    PairScalars<double, (T <= 128)> ps;
     double* Sh = (double*)hist;
-    const int code = run_phase<T, A, P64, 0>(tm, n, x64, g, f, Sh, Sh + hstride, rho, gmv, sup, cnt,
+    const int code = run_phase<T, A, P64, 0>(tm, n, x64, g, f, Sh, Sh + hstride, ps, cnt,
                                                  head, iters, r.evals64, r.iters64, r.vec64, pos,
                                                  hbuf, p, t0, cyc);
     r.E = f;
@@ -1499,7 +1480,7 @@ __device__ __forceinline__ void minimise(const Team<T>& tm, int n, double (&x64)
   } else {
     float* Sh = (float*)hist;
     float* Yh = Sh + hstride;
-    float rho[LJ_MAX_M], gmv[LJ_MAX_M], sup[LJ_MAX_M];
+    PairScalars<float, (T <= 128)> ps;
     int code = PH_SWITCH;
     float dummy32;
     // ---- tier 1: FP32 -------------------------------------------------------
@@ -1516,7 +1497,7 @@ __device__ __forceinline__ void minimise(const Team<T>& tm, int n, double (&x64)
       r.evals32 = 1;
       const float gm = grad_max<T, A, float>(tm, g32);
       if (fisfinite(f32) && gm < __int_as_float(0x7f800000) && !(gm < (float)p.switch_gtol)) {
-        code = run_phase<T, A, P32, 1>(tm, n, x32, g32, f32, Sh, Yh, rho, gmv, sup, cnt, head,
+        code = run_phase<T, A, P32, 1>(tm, n, x32, g32, f32, Sh, Yh, ps, cnt, head,
                                            iters, r.evals32, r.iters32, r.vec32, pos, nullptr, p,
                                            t0, cyc);
         moved32 = r.iters32 > 0;
@@ -1552,7 +1533,7 @@ __device__ __forceinline__ void minimise(const Team<T>& tm, int n, double (&x64)
           need_fp64 = true;               // confirm (and finish) in FP64
           break;
         }
-        code = run_phase<T, A, PDF, 2>(tm, n, xdf, gdf, fdf, Sh, Yh, rho, gmv, sup, cnt, head, iters,
+        code = run_phase<T, A, PDF, 2>(tm, n, xdf, gdf, fdf, Sh, Yh, ps, cnt, head, iters,
                                           r.evals_df, r.iters64, r.vec64, pos, hbuf, p, t0, cyc);
         if (code == PH_CONVERGED) {
           gm = 0.f;
@@ -1581,7 +1562,7 @@ __device__ __forceinline__ void minimise(const Team<T>& tm, int n, double (&x64)
       if (gm < p.gtol) {
         r.E = f; r.iters = iters; r.status = ST_CONVERGED; lap(r.cyc64); return;
       }
-      code = run_phase<T, A, P64m, 0>(tm, n, x64, g, f, Sh, Yh, rho, gmv, sup, cnt, head, iters,
+      code = run_phase<T, A, P64m, 0>(tm, n, x64, g, f, Sh, Yh, ps, cnt, head, iters,
                                           r.evals64, r.iters64, r.vec64, pos, hbuf, p, t0, cyc);
       r.E = f;
       r.iters = iters;

@@ -68,14 +68,7 @@ static_assert(sizeof(PosDG<2>) == 48 && sizeof(PosDG<4>) == 96 && sizeof(SlotF<4
 // the first warp in a fixed order: L lanes a candidate, strided, then a tree
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void acc_pair(ff& s, ff v) { df_acc(s, v); }
-// TwoSum with the operands ordered by magnitude on the integer pipe: three
-// FP64 additions (Dekker's FastTwoSum) instead of six
-__device__ __forceinline__ void acc_pair(dd& s, dd v) {
-  const bool sw = (__double2hiint(s.hi) & 0x7fffffff) < (__double2hiint(v.hi) & 0x7fffffff);
-  const double a = sw ? v.hi : s.hi, b = sw ? s.hi : v.hi;
-  s.hi = __dadd_rn(a, b);
-  s.lo = __dadd_rn(s.lo, __dadd_rn(__dsub_rn(b, __dsub_rn(s.hi, a)), v.lo));
-}
+__device__ __forceinline__ void acc_pair(dd& s, dd v) { dd_acc(s, v); }
 __device__ __forceinline__ double total(ff s) { return (double)s.hi + (double)s.lo; }
 __device__ __forceinline__ double total(dd s) { return __dadd_rn(s.hi, s.lo); }
 

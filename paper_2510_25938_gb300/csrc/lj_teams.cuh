@@ -25,19 +25,29 @@ __host__ __device__ constexpr int cta_threads_for(int T) { return T < 128 ? 128 
 
 __host__ __device__ constexpr size_t align16(size_t b) { return (b + 15) & ~size_t(15); }
 
-// Half-pair buffers (24 bytes per pair) are used for clusters of up to
-// kHalfMaxN atoms; teams for more than kTileMinN atoms hold the
-// double-float tile accumulators (24 bytes per atom) in the same slot; in
-// between, double-float evaluations are one-sided (measured: with 3 to 8
-// atom blocks a tile round leaves warps idle).
+// How FP64 and double-float evaluations take every pair once, by the largest
+// cluster of the launch, and the team's buffer for it:
+//   up to kHalfMaxN atoms    half pairs, 24 bytes per pair;
+//   up to kTileMinN          ring, 24 bytes per atom and shift of a chunk (4,096
+//                            clusters of 13..150 atoms, mixed: 17.1 ms, 19.1 with
+//                            one-sided rows, which evaluate every pair twice; 3
+//                            to 8 atom blocks leave warps idle in a tile round);
+//   above                    32 x 32 tiles, 24 bytes per atom.
 constexpr int kHalfMaxN = 64;
 constexpr int kTileMinN = 256;
+enum PairLayout : int { LAYOUT_HALF = 0, LAYOUT_TILES = 1, LAYOUT_RING = 2 };
+__host__ __device__ constexpr int pair_layout(int max_n) {
+  return max_n <= kHalfMaxN ? LAYOUT_HALF : max_n <= kTileMinN ? LAYOUT_RING : LAYOUT_TILES;
+}
+// shifts of a ring chunk: the history of up to 256 atoms (m = 10, FP32) stays
+// on chip beside it
+__host__ __device__ constexpr int ring_shifts(int max_n) { return max_n <= 128 ? 8 : 4; }
 
 __host__ __device__ constexpr size_t half_bytes(int max_n, bool half) {
   return !half ? 0
-         : max_n <= kHalfMaxN ? align16((size_t)24 * (max_n * (max_n - 1) / 2))
-         : max_n > kTileMinN  ? align16((size_t)24 * max_n)
-                              : 0;
+         : align16((size_t)24 * (pair_layout(max_n) == LAYOUT_HALF   ? max_n * (max_n - 1) / 2
+                                 : pair_layout(max_n) == LAYOUT_RING ? max_n * ring_shifts(max_n)
+                                                                     : max_n));
 }
 
 // per-team shared bytes: positions (32-byte records; the FP32 phase uses the
@@ -65,6 +75,11 @@ __device__ __forceinline__ void carve_team(unsigned char* base, int max_n, bool 
   p += (T > 32 ? 2 * 8 * (T / 32) * sizeof(double) : 0);
   word = reinterpret_cast<long long*>(p);
 }
+
+// What a kernel is allowed to ask for: the most a CTA can have (227 KB), set
+// once and for all its launches -- the buckets of one call share kernels, and a
+// smaller value set for one would refuse the launch of another.
+constexpr int kSmemMax = 227 * 1024;
 
 // History goes on chip when a CTA's shared memory stays within this budget.
 constexpr size_t kSmemBudget = 100 * 1024;
