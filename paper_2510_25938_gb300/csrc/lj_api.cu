@@ -53,7 +53,8 @@ struct DeviceGuard {
   bool ok = false;
   explicit DeviceGuard(int dev) {
     if (cudaGetDevice(&prev) != cudaSuccess) prev = -1;
-    ok = cudaSetDevice(dev) == cudaSuccess;
+    ok = prev == dev || cudaSetDevice(dev) == cudaSuccess;
+    if (prev == dev) prev = -1;          // nothing to restore
   }
   ~DeviceGuard() {
     if (prev >= 0) cudaSetDevice(prev);
@@ -390,6 +391,7 @@ lj_status lj_energy_grad_batched_pot(lj_ctx* ctx, const lj_batch* batch, lj_prec
   a.energy = d_energy;
   a.grad = d_grad;
   a.k = ljh::make_consts(eps, sigma, potential, rho);
+  a.sms = ctx->sms;
   cudaError_t e = ljh::eval_launch(a, (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "lj_energy_grad_batched launch");
   return LJ_OK;

@@ -455,11 +455,7 @@ cudaError_t launch_io(const ljh::EvalArgs& a, int sms, cudaStream_t s) {
 namespace ljh {
 
 cudaError_t eval_launch(const EvalArgs& a, cudaStream_t s) {
-  int dev = 0, sms = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e != cudaSuccess) return e;
-  return a.xtype == LJ_F32 ? launch_io<float>(a, sms, s) : launch_io<double>(a, sms, s);
+  return a.xtype == LJ_F32 ? launch_io<float>(a, a.sms, s) : launch_io<double>(a, a.sms, s);
 }
 
 }  // namespace ljh

@@ -32,6 +32,7 @@ struct EvalArgs {
   double* energy;
   void* grad;
   LjConsts k;           // pair-potential constants (Eq. (1) or Morse)
+  int sms;              // SMs of the device
 };
 
 struct LbfgsArgs {

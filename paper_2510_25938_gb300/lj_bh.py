@@ -90,6 +90,8 @@ def library_path() -> str:
 def load():
     """Load liblj_bh.so; raises if it is missing (build it with build.build())."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             if not os.path.exists(_build.LIB):
@@ -138,7 +140,7 @@ def load():
             lib.lj_ctx_autotune_bh.argtypes = [P, C.POINTER(_State), C.POINTER(_Bh),
                                                C.POINTER(_Tuning), P]
             lib.lj_ctx_autotune_bh.restype = C.c_int
-            _lib = lib
+            _lib = lib          # last: load() reads it without the lock
     return _lib
 
 
@@ -154,7 +156,8 @@ def _ptr(t) -> int | None:
 
 def _stream(stream) -> int | None:
     if stream is None:
-        stream = torch.cuda.current_stream()
+        # torch.cuda.current_stream().cuda_stream without building a Stream object
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     return stream.cuda_stream
 
 
