@@ -379,8 +379,11 @@ RingLaunch ring_plan(const ljh::EvalArgs& a, int sms) {
     pl.P = (int)std::max(1LL, std::min<long long>(std::min(more, (long long)NG / 2 + 1), kRingMaxB / NG));
     r.B = (NG * pl.P + 31) / 32 * 32;
   } else {
-    // uneven: one candidate a CTA, its parts set by the kernel from its own size
-    r.B = std::max(128, (NG + 31) / 32 * 32);
+    // uneven: one candidate a CTA, its parts set by the kernel from its own
+    // size; small candidates cannot use many threads (6,583 of 8..47 atoms, FP32
+    // Morse: 25 us a call with one warp, 44 us with 128 threads; 4,096 of 13..150
+    // atoms, FP32: 44 us with 128 threads, 45 with 64, 57 with 32)
+    r.B = NG <= 13 ? 32 : NG <= 26 ? 64 : std::max(128, (NG + 31) / 32 * 32);
     pl.P = 2;                                // (reserves the parts' buffer)
   }
   const int H = NG / 2;
