@@ -12,11 +12,16 @@ using namespace ljd;
 using namespace ljr;
 
 // ---- FP32 --------------------------------------------------------------------
-// MULTI = false: one part, one CTA per candidate, all H shifts before one
-// barrier (large uniform batches of small clusters).  MULTI = true: any batch.
-template <int G, typename IO, int POT, bool SIG, bool MULTI>
+// PACKED: C candidates a CTA, one part each, all H shifts before one barrier
+// (large uniform batches of small clusters).  PACKED_UNEVEN: the same, every
+// candidate with the threads of the largest; a variant of its own, since its
+// sizes and bounds cost PACKED 6% (65,536 x LJ38: 61.1 against 57.4 us).
+// MULTI_PART: any batch.
+enum RingMode { PACKED, PACKED_UNEVEN, MULTI_PART };
+template <int G, typename IO, int POT, bool SIG, int MODE>
 __global__ void __launch_bounds__(256, 2) eval_ring_f32_kernel(ljh::EvalArgs a, RingPlan pl) {
   extern __shared__ __align__(16) unsigned char smem[];
+  constexpr bool MULTI = MODE == MULTI_PART, UNEVEN = MODE == PACKED_UNEVEN;
   const int B = blockDim.x, tid = threadIdx.x;
   const int S = MULTI ? pl.S : 1, KS = pl.KS;
   PosRing<G>* pos = reinterpret_cast<PosRing<G>*>(smem);
@@ -43,14 +48,30 @@ __global__ void __launch_bounds__(256, 2) eval_ring_f32_kernel(ljh::EvalArgs a, 
     p = P > 1 ? rem / NG : 0;
     g = rem - p * NG;
   };
-  if (a.uniform_n > 0) {
+  const int NS = UNEVEN ? (a.max_n + G - 1) / G : NG;   // packed: threads of a candidate
+  if (UNEVEN) {
+    lc = tid / NS;
+    g = tid - lc * NS;
+  } else if (a.uniform_n > 0) {
     P = MULTI ? pl.P : 1;
     place();
   }
   for (long long c0 = (long long)(blockIdx.x / S) * pl.C; c0 < a.n_cand; c0 += stride) {
     long long a0;
-    if (!MULTI || a.uniform_n > 0) {
+    bool bad = false;
+    if (MODE == PACKED || (MULTI && a.uniform_n > 0)) {
       a0 = (c0 + lc) * n;
+    } else if (UNEVEN) {
+      n = 0;
+      a0 = 0;
+      if (lc < pl.C && c0 + lc < a.n_cand) {
+        a0 = a.off[c0 + lc];
+        const long long na = a.off[c0 + lc + 1] - a0;
+        bad = na > a.max_n || na < 0;
+        n = bad ? 0 : (int)na;
+      }
+      NG = (n + G - 1) / G;
+      H = NG >> 1;
     } else {
       a0 = a.off[c0];
       n = (int)(a.off[c0 + 1] - a0);
@@ -63,9 +84,10 @@ __global__ void __launch_bounds__(256, 2) eval_ring_f32_kernel(ljh::EvalArgs a, 
       P = NG > 0 ? max(1, min(B / NG, (H + S - 1) / S + 1)) : 1;
       place();
     }
-    const bool live = lc < pl.C && c0 + lc < a.n_cand;
-    const int slot = (lc * P + p) * NG;      // first slot of this candidate's part
-    const int pslot = lc * NG;               // its first position record
+    const bool here = lc < pl.C && c0 + lc < a.n_cand;
+    const bool live = here && (!UNEVEN || g < NG);
+    const int slot = UNEVEN ? lc * NS : (lc * P + p) * NG;  // first slot of this candidate's part
+    const int pslot = UNEVEN ? slot : lc * NG;              // its first position record
     V2 N[G / 2];                             // own atoms, negated
     {
       float q[3 * G];
@@ -99,8 +121,10 @@ __global__ void __launch_bounds__(256, 2) eval_ring_f32_kernel(ljh::EvalArgs a, 
           shift<G, POT, SIG>(N, pos[pslot + t], even && k == H, g < H, k0, k1, o, e,
                              react[s * B + slot + t]);
         }
-        es[tid] = e;
+        if (!UNEVEN) es[tid] = e;
       }
+      // zeros from a candidate's idle threads, NaN for a bad size
+      if (UNEVEN && here) es[tid] = bad && g == 0 ? ff{__int_as_float(0x7fc00000), 0.f} : e;
       __syncthreads();
       if (live && (MULTI || gout)) {
         for (int s = 0; s < KS; ++s) {
@@ -117,7 +141,7 @@ __global__ void __launch_bounds__(256, 2) eval_ring_f32_kernel(ljh::EvalArgs a, 
         for (int pp = 1; pp < P; ++pp) own_slot<true>(o, own[slot + pp * NG + g]);
     }
     if (tid < 32)
-      sum_energies(es, pl.C, NG * P, [&](int c, ff s) {
+      sum_energies(es, pl.C, UNEVEN ? NS : NG * P, [&](int c, ff s) {
         if (MULTI && S > 1) ecl[c] = s;
         else if (c0 + c < a.n_cand) a.energy[c0 + c] = total(s) * ef;
       });
@@ -378,6 +402,13 @@ RingLaunch ring_plan(const ljh::EvalArgs& a, int sms) {
     const long long more = want / (a.n_cand * NG);
     pl.P = (int)std::max(1LL, std::min<long long>(std::min(more, (long long)NG / 2 + 1), kRingMaxB / NG));
     r.B = (NG * pl.P + 31) / 32 * 32;
+  } else if (fp32 && NG / 2 <= ring_most_ks(4, false) && 2 * a.n_cand * NG > want) {
+    // large uneven batch of small clusters: packed like a uniform one, every
+    // candidate with the threads of the largest (33,563 of 4..9 atoms: 22 us a
+    // call, 55 with a CTA each)
+    r.B = 64;
+    pl.C = r.B / NG;
+    r.multi = false;
   } else {
     // uneven: one candidate a CTA, its parts set by the kernel from its own
     // size; small candidates cannot use many threads (6,583 of 8..47 atoms, FP32
@@ -441,9 +472,11 @@ cudaError_t launch_typed(const ljh::EvalArgs& a, int sms, cudaStream_t s) {
     if (r.G == 3) return launch_ring(eval_ring_f64_kernel<3, IO, POT, SIG>, a, r, s);
     return launch_ring(eval_ring_f64_kernel<4, IO, POT, SIG>, a, r, s);
   }
-  if (r.multi) return launch_ring(eval_ring_f32_kernel<4, IO, POT, SIG, true>, a, r, s);
-  return r.G == 8 ? launch_ring(eval_ring_f32_kernel<8, IO, POT, SIG, false>, a, r, s)
-                  : launch_ring(eval_ring_f32_kernel<4, IO, POT, SIG, false>, a, r, s);
+  if (r.multi) return launch_ring(eval_ring_f32_kernel<4, IO, POT, SIG, MULTI_PART>, a, r, s);
+  if (a.uniform_n <= 0)
+    return launch_ring(eval_ring_f32_kernel<4, IO, POT, SIG, PACKED_UNEVEN>, a, r, s);
+  return r.G == 8 ? launch_ring(eval_ring_f32_kernel<8, IO, POT, SIG, PACKED>, a, r, s)
+                  : launch_ring(eval_ring_f32_kernel<4, IO, POT, SIG, PACKED>, a, r, s);
 }
 
 template <typename IO>

@@ -94,7 +94,8 @@ def test_eval_ring_uniform(lj, n, n_cand, f32, morse):
 
 
 @pytest.mark.parametrize("f32,morse", [(True, False), (False, False), (True, True), (False, True)])
-@pytest.mark.parametrize("lo,hi,n_cand", [(0, 20, 70), (2, 150, 60), (90, 400, 12), (500, 1024, 3)])
+@pytest.mark.parametrize("lo,hi,n_cand", [(0, 20, 70), (2, 150, 60), (90, 400, 12), (500, 1024, 3),
+                                          (0, 9, 14000), (3, 52, 5000)])
 def test_eval_ring_uneven(lj, lo, hi, n_cand, f32, morse):
     sizes = I.uneven_sizes(n_cand, lo, hi, hi)
     sizes[-1] = hi
@@ -104,6 +105,25 @@ def test_eval_ring_uneven(lj, lo, hi, n_cand, f32, morse):
         x = x.astype(np.float32).astype(np.float64)
     e, g = _evaluate(lj, x, n_cand, hi, off, f32, morse, 0)
     _check(x, off, e, g, f32, morse)
+
+
+@pytest.mark.parametrize("f32", [True, False])
+@pytest.mark.parametrize("n_cand", [50, 12000])
+def test_eval_ring_bad_size(lj, n_cand, f32):
+    """A candidate above max_n gets a NaN energy and no gradient; the others are
+    what they are without it."""
+    sizes = np.full(n_cand, 5)
+    sizes[7] = 12
+    off = I.offsets_from_sizes(sizes)
+    x = np.concatenate([_starts(int(k), 1, i) for i, k in enumerate(sizes)])
+    if f32:
+        x = x.astype(np.float32).astype(np.float64)
+    e, g = _evaluate(lj, x, n_cand, 9, off, f32, False, 0)
+    assert np.isnan(e[7]) and (g[3 * off[7]:3 * off[8]] == 7.0).all()
+    keep = np.r_[0:7, 8:n_cand]
+    xs = np.concatenate([x[3 * off[c]:3 * off[c + 1]] for c in keep])
+    gs = np.concatenate([g[3 * off[c]:3 * off[c + 1]] for c in keep])
+    _check(xs, np.arange(keep.size + 1) * 5, e[keep], gs, f32, False)
 
 
 @pytest.mark.parametrize("n", [38, 40, 100])
