@@ -265,8 +265,7 @@ lj_status lj_energy_grad_batched(lj_ctx* ctx, const lj_batch* batch, lj_precisio
  * gives exactly lj_energy_grad_batched (eps, sigma; rho unused);
  * LJ_POT_MORSE evaluates E = eps sum_{i<j} e (e - 2), e = exp(rho (1 - r/re)),
  * with re = sigma, and its gradient dE/dx_i = -(2 eps rho / re) sum_{j != i}
- * e (e - 1) (x_i - x_j) / r_ij.  Morse clusters run one team per candidate
- * in one-sided rows, FP32 (FP32 exp and reciprocal square root,
+ * e (e - 1) (x_i - x_j) / r_ij, FP32 (FP32 exp and reciprocal square root,
  * compensated energy) or FP64.  Errors as lj_energy_grad_batched, plus
  * INVALID_ARG for an unknown potential or rho outside (0, 64] (Morse).
  */

@@ -87,40 +87,6 @@ __device__ __forceinline__ V team_sum1(const Team<T>& tm, V x) {
   return v[0];
 }
 
-// Max over the team (inputs are >= 0; a non-finite entry must be passed as +inf).
-template <int T, int NV, typename V>
-__device__ __forceinline__ void team_max(const Team<T>& tm, V (&v)[NV]) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-    for (int k = 0; k < NV; ++k) v[k] = fmax(v[k], shfl_xor(v[k], o));
-  }
-  if constexpr (T > 32) {
-    constexpr int NW = T / 32;
-    V* buf = reinterpret_cast<V*>(tm.scratch());
-    if ((tm.rank & 31) == 0) {
-#pragma unroll
-      for (int k = 0; k < NV; ++k) buf[(tm.rank >> 5) * NV + k] = v[k];
-    }
-    tm.sync();
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      V s = buf[k];
-#pragma unroll
-      for (int w = 1; w < NW; ++w) s = fmax(s, buf[w * NV + k]);
-      v[k] = s;
-    }
-  }
-}
-
-// |x| with NaN mapped to +inf, so that fmax-based norms flag non-finite input
-__device__ __forceinline__ float abs_nan_inf(float x) {
-  return (x != x) ? __int_as_float(0x7f800000) : fabsf(x);
-}
-__device__ __forceinline__ double abs_nan_inf(double x) {
-  return (x != x) ? __longlong_as_double(0x7ff0000000000000LL) : fabs(x);
-}
-
 // ---------------------------------------------------------------------------
 // Float-float energy values (FP32 phase): hi + lo, |lo| <= ulp(hi)/2.
 // The FP32 phase keeps its energies in this form so that the line search can
@@ -432,10 +398,8 @@ __device__ __forceinline__ void stage_f32x2(PosF2* pos, int n, int i, float x, f
 // `pos`: b = sum_j c_ij (x_j - x_i) with c = s2 s6 (2 s6 - 1), s2 = sigma^2
 // / r^2 (SIG: sigma != 1, sig2 = sigma^2), and e += sum_j s6 (s6 - 1), the
 // self term excluded.  Energy: per lane, blocks of 4 terms summed in FP32,
-// the two lanes' block sums added and folded into the float-float `e`
-// (FF), or summed in plain FP32 into e.hi (!FF: ~8 ulps of the row, below the
-// pair terms' own error; used where the energy is only reported).
-template <bool SIG, bool FF = true>
+// the two lanes' block sums added and folded into the float-float `e`.
+template <bool SIG>
 __device__ __forceinline__ void pair_row_f32x2(int n, int i, float px, float py, float pz,
                                                const PosF2* __restrict__ pos, float sig2,
                                                float& bx, float& by, float& bz, ff& e) {
@@ -468,14 +432,12 @@ __device__ __forceinline__ void pair_row_f32x2(int n, int i, float px, float py,
     float2 eb = f2(0.f);
 #pragma unroll
     for (int u = 0; u < 4; ++u) term(m + u, eb);
-    if constexpr (FF) e = ff_add_f(e, __fadd_rn(eb.x, eb.y));
-    else e.hi = __fadd_rn(e.hi, __fadd_rn(eb.x, eb.y));
+    e = ff_add_f(e, __fadd_rn(eb.x, eb.y));
   }
   if (m < M) {
     float2 eb = f2(0.f);
     for (; m < M; ++m) term(m, eb);
-    if constexpr (FF) e = ff_add_f(e, __fadd_rn(eb.x, eb.y));
-    else e.hi = __fadd_rn(e.hi, __fadd_rn(eb.x, eb.y));
+    e = ff_add_f(e, __fadd_rn(eb.x, eb.y));
   }
   bx = __fadd_rn(ax.x, ax.y);
   by = __fadd_rn(ay.x, ay.y);
@@ -688,7 +650,6 @@ __device__ __forceinline__ ff df_from_double(double x) {
   const float h = (float)x;
   return ff{h, (float)(x - (double)h)};
 }
-__device__ __forceinline__ double df_to_double(ff a) { return (double)a.hi + (double)a.lo; }
 
 // |d|^2 of a double-float vector (not necessarily normalised) with one
 // renormalisation: the high squares exactly (TwoProd by FMA), summed by two

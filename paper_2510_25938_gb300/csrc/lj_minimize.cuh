@@ -84,16 +84,6 @@ struct Prec {
   using S = std::conditional_t<sizeof(V_) == 8, double, float>;
   using F = std::conditional_t<std::is_same<XP_, double>::value, double, ff>;
 };
-using PrecF32 = Prec<float, float, float, 0>;      // mixed: FP32 tier
-using PrecDF = Prec<ff, float, float, 1>;          // mixed: double-float tier
-using PrecF64m = Prec<double, double, float, 0>;   // mixed: FP64 tier
-using PrecF64 = Prec<double, double, double, 0>;   // FP64 path
-
-// Eval-only helper: scalars of a plain single-precision evaluation.
-template <typename X> struct Tr;
-template <> struct Tr<float> { using S = float; using F = ff; };
-template <> struct Tr<double> { using S = double; using F = double; };
-
 // trial position x + a d and step xt - x for each position type
 __device__ __forceinline__ float pos_step(float x, float a, float d) { return x + a * d; }
 template <typename SA, typename VD>
@@ -138,15 +128,13 @@ __device__ __forceinline__ int hidx(int slot, int a, int c, int rank) {
 // ---------------------------------------------------------------------------
 // Morse pair potential (Morse 1929, cluster form), the pair-potential
 // extension of the method: V(r) = eps e (e - 2), e = exp(rho (1 - r / re)),
-// re in the sigma slot.  One-sided rows: every thread sums, for each atom it
-// owns, the terms of all other atoms (deterministic, no shared pair buffer);
+// re in the sigma slot.  FP32 (and FP64 without a pair buffer) in one-sided rows:
+// every thread sums, for each atom it owns, the terms of all other atoms;
 // E = (eps / 2) sum_i sum_{j != i} e (e - 2), and
 // g_i = -(2 eps rho / re) sum_{j != i} e (e - 1) (x_i - x_j) / r.
 // FP32 (first tier of the mixed path; compensated energy), double-float
-// (evaluate_morse_df, the polish tier) and FP64.  FP64 teams with
-// a half-pair buffer (clusters of up to 64 atoms) take each pair once, as
-// for Eq. (1): pair p's vector e (e - 1) (x_i - x_j) / r goes to the buffer,
-// then every (atom, component) row is summed, +v over j > i, -v over j < i.
+// (evaluate_morse_df, the polish tier) and FP64; those two take each pair once
+// through the team's buffer up to 256 atoms, as for Eq. (1) (half pairs, ring).
 // Coincident atoms give E = +inf (and a non-finite gradient), as for Eq. (1).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ float to_value(ff v) { return v.hi + v.lo; }
@@ -181,8 +169,8 @@ __device__ __forceinline__ void pair_term_morse_f64(const PosD& a, const PosD& b
 
 // Double-float Morse evaluation (the mixed path's polish tier): positions
 // scaled by 1/re, pair terms by pair_term_morse_df (double-float exponential
-// and square root); each pair once through the half-pair buffer for clusters
-// of up to 64 atoms, one-sided rows above.
+// and square root); each pair once through the team's buffer up to 256 atoms
+// (half pairs, ring), one-sided rows above.
 template <int T, int A, typename P>
 __device__ __forceinline__ void evaluate_morse_df(const Team<T>& tm, int n,
                                                   const typename P::XP (&x)[A][3],
@@ -745,7 +733,7 @@ __device__ __forceinline__ S cubic_step(S a, F fa, S ga, S b, F fb, S gb) {
 // ---------------------------------------------------------------------------
 // Two-loop recursion by the team's first warp (teams of 1 to 4 warps; float
 // history staged through the idle position buffer, FP64 history through the
-// idle half-pair buffer).  The recursion is a chain of 2 cnt + 1 dependent inner products;
+// idle pair buffer).  The recursion is a chain of 2 cnt + 1 dependent inner products;
 // done by the whole team, each one crosses warps through shared memory and a
 // barrier.  Instead every thread stages its gradient in `xb` (the idle
 // position buffer, 12 A T + 4 bytes), warp 0 runs the recursion over all T
@@ -1068,7 +1056,7 @@ __device__ __forceinline__ int run_phase(const Team<T>& tm, int n, typename P::X
     bool led = false;
     if constexpr (T <= 128) {
       // staging buffer for the lead warp: the idle position buffer (32 n
-      // bytes) for float history, the idle half-pair buffer (24 bytes per
+      // bytes) for float history, the idle pair buffer (half pairs: 24 bytes per
       // pair) for double history
       V* xb = nullptr;
       if constexpr (std::is_same<V, float>::value) {
