@@ -328,14 +328,17 @@ __device__ __forceinline__ float ex2_approx(float x) {
   return r;
 }
 
-// 1 / a in FP64: the hardware's estimate r (PTX rcp.approx.ftz.f64, ~2^-20
-// relative) and one third-order Householder step, r (1 + e + e^2) with
-// e = 1 - a r formed by one FMA: the truncation error e^3 is below 2^-58, so the
-// result is within an ulp of 1 / a.  Three FP64 instructions, against about
-// nine of the correctly rounded reciprocal, and none on the FP64 pipe for the
-// ends of the range: an estimate of 0 or infinity (a = 0, infinite or so small
-// that its inverse overflows) is returned as it is, chosen by its exponent
-// bits on the integer pipe.
+// 1 / a in FP64, correctly rounded: the hardware's estimate r (PTX
+// rcp.approx.ftz.f64, ~2^-20 relative), one third-order Householder step,
+// y = r (1 + e + e^2) with e = 1 - a r formed by one FMA (truncation error
+// e^3 < 2^-58: within an ulp), and Markstein's correction y + y (1 - a y)
+// (IBM J. Res. Dev. 34, 1990), whose residual is exact and whose own error is far
+// below the distance of any 1 / a from a rounding boundary, but for the
+// significand of all ones.  Five FP64 instructions, about nine of __drcp_rn
+// (65,536 x LJ38: 2.23 ms; 2.07 without the correction, which leaves a few results
+// in a thousand an ulp off).  None on the FP64 pipe for the ends of the range: an estimate of 0 or infinity (a = 0, infinite
+// or so small that its inverse overflows) is returned as it is, chosen by its
+// exponent bits on the integer pipe.
 __device__ __forceinline__ bool f64_end(double r) {   // 0, subnormal, infinite or NaN
   const int ex = __double2hiint(r) & 0x7ff00000;
   return ex == 0 || ex == 0x7ff00000;
@@ -344,7 +347,8 @@ __device__ __forceinline__ double rcp_f64(double a, double one = 1.0) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
   const double e = fma(-a, r, one);
-  const double y = fma(r, fma(e, e, e), r);
+  double y = fma(r, fma(e, e, e), r);
+  y = fma(y, fma(-a, y, one), y);
   return f64_end(r) ? r : y;
 }
 // 1 / sqrt(a) in FP64, likewise: with e = 1 - a r^2, r (1 + e/2 + 3 e^2 / 8)
@@ -765,22 +769,30 @@ __device__ __forceinline__ void pair_row_df(int n, int i, ff px, ff py, ff pz,
 }
 
 // ---------------------------------------------------------------------------
-// Half-pair evaluation (FP64 and double-float, clusters of up to 64 atoms):
-// each unordered pair once, in the order of a ring: pair p is atom i = p mod n
-// with j = (i + k) mod n, k = 1 + p / n (for even n the shift n/2 holds the n/2
-// pairs i < n/2).  Thread p mod T evaluates it and writes its vector
+// Half-pair evaluation (FP64 and double-float, clusters of up to 64 atoms): each
+// unordered pair once.  Thread p mod T evaluates pair p and writes its vector
 // v_p = c_ij (x_i - x_j) to a shared buffer; after a barrier the sum of an atom
-// and axis takes +v of the pairs that start at the atom, ((k-1) n + atom), and
-// -v of those that end there, ((k-1) n + (atom - k) mod n).  Both run through
-// the buffer with consecutive lanes at consecutive words: no bank conflicts and
-// one index and one comparison a term, where the triangular order took a
-// select of two row bases, a select of the sign and eight-byte strides of a
-// whole row.  Every pair costs one evaluation instead of two and the work
+// and axis takes +v of the pairs that start at the atom and -v of those that
+// end there.  Every pair costs one evaluation instead of two and the work
 // splits evenly over the team whatever N is.  Fixed pair order, fixed sum order.
+//
+// Mixed precision (double-float and its FP64 tier): the order of a ring.  Pair p is atom i = p mod n with
+// j = (i + k) mod n, k = 1 + p / n (for even n the shift n/2 holds the n/2 pairs
+// i < n/2), so that an atom's pairs are at ((k-1) n + atom) and
+// ((k-1) n + (atom - k) mod n): consecutive lanes at consecutive words, no bank
+// conflicts, one index and one comparison a term.
+//
+// FP64 path: row-major order of the upper triangle, i < j, and row sums over j = 0 ..
+// n-1 in four interleaved parts.  Which order is taken shows in results: at the
+// default gtol of 1e-6 the decrease that a last line search has to resolve
+// (~1e-15 for LJ13) is below an ulp of E, so whether a trial ends as CONVERGED
+// or as LINESEARCH_FAIL is decided by the last bit of a sum, and a Basin Hopping
+// trace records it.  The ring's order with a flat history and a reciprocal within
+// an ulp is faster (50 steps of LJ13: 37 against 46 ms) but gives other traces.
 // ---------------------------------------------------------------------------
 __host__ __device__ constexpr int n_pairs(int n) { return n * (n - 1) / 2; }
 
-// pair (i, j) of index p, advanced by a fixed step
+// pair (i, j) of index p in the ring's order, advanced by a fixed step
 struct PairWalk {
   int i, k;
   __device__ __forceinline__ PairWalk(int n, int p) : i(p % n), k(1 + p / n) {}
@@ -868,6 +880,84 @@ __device__ __forceinline__ void half_rows(int rank, int n, const F* vb, G scale,
       else half_minus(s3, vc[ii - n / 2]);
     }
     sums[3 * ii + axis] = scale * half_total(s0, s1, s2, s3);
+  }
+}
+
+// pair (i, j) of index p, i < j, in the row-major upper triangle; j = -1 if none
+struct TriWalk {
+  int i, j;
+  __device__ __forceinline__ TriWalk(int n, int p) : i(0) {
+    int row = n - 1;
+    while (row > 0 && p >= row) { p -= row; ++i; --row; }
+    j = row > 0 ? i + 1 + p : -1;
+  }
+  __device__ __forceinline__ void advance(int n, int step) {
+    j += step;
+    while (i < n - 1 && j >= n) {
+      j -= n;         // j - n = offset past the row end
+      ++i;
+      j += i + 1;     // first column of the next row is i+1
+    }
+  }
+};
+// pair (j, i), j < i, sits at tri_base(n, j) + i and pair (i, j), j > i, at
+// tri_base(n, i) + j; tri_base(n, j + 1) = tri_base(n, j) + n - j - 2,
+// tri_base(n, 0) = -1
+__device__ __forceinline__ int tri_base(int n, int i) {
+  return i * (2 * n - i - 1) / 2 - i - 1;
+}
+
+// two pairs in flight a thread, as half_pairs; the energies of the two are
+// added in FP64, then to the double-double sum
+template <int T, typename Term>
+__device__ __forceinline__ void tri_pairs(int rank, int n, double* vb, Term&& term, dd& e) {
+  const int np = n_pairs(n);
+  TriWalk w1(n, rank), w2 = w1;
+  w2.advance(n, T);
+  for (int q = rank; q < np; q += 2 * T) {
+    const bool two = q + T < np;
+    double ax, ay, az, ae, bx, by, bz, be;
+    term(w1.i, w1.j, ax, ay, az, ae);
+    term(two ? w2.i : 0, two ? w2.j : 1, bx, by, bz, be);
+    vb[q] = ax; vb[np + q] = ay; vb[2 * np + q] = az;
+    double eb = ae;
+    if (two) {
+      vb[q + T] = bx; vb[np + q + T] = by; vb[2 * np + q + T] = bz;
+      eb += be;
+    }
+    dd_acc(e, eb);
+    w1.advance(n, 2 * T);
+    w2.advance(n, 2 * T);
+  }
+}
+
+// sums[3 atom + axis] = -gs * sum, one (atom, axis) a thread; all lanes walk j
+// together, +v over j > atom, -v over j < atom
+template <int T>
+__device__ __forceinline__ void tri_rows(int rank, int n, const double* vb, double gs,
+                                              double* sums) {
+  const int np = n_pairs(n);
+  for (int q3 = rank; q3 < 3 * n; q3 += T) {
+    const int ii = q3 / 3;
+    const double* vc = vb + (q3 - 3 * ii) * np;
+    const int ri = tri_base(n, ii);
+    int rj = -1;                           // tri_base(n, j)
+    double s[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int j0 = 0; j0 < n; j0 += 4) {
+      double v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int j = j0 + u;
+        const int q = j < ii ? rj + ii : ri + j;
+        v[u] = 0.0;
+        if (j < n && j != ii) v[u] = vc[q];
+        if (j < ii) v[u] = -v[u];
+        rj += n - j - 2;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) s[u] += v[u];
+    }
+    sums[q3] = -gs * ((s[0] + s[1]) + (s[2] + s[3]));
   }
 }
 

@@ -52,10 +52,11 @@ __global__ void __launch_bounds__(cta_threads_for(T), min_ctas(T, A, MIXED))
   void* hbuf;
   void* hist;
   const size_t hb = a.hist_on_chip ? a.hist_slot_bytes : 0;
-  carve_team<T>(smem + team * team_smem_bytes<T>(a.max_n, true, hb), a.max_n, true, hb, pos,
-                hbuf, hist, tm.red, word);
+  const bool buf = pair_buffer(a.max_n, MIXED);
+  carve_team<T>(smem + team * team_smem_bytes<T>(a.max_n, buf, hb), a.max_n, buf, hb, pos, hbuf,
+                hist, tm.red, word);
   MinParams p = to_dev(a.p);
-  // hbuf: pairs up to 64 atoms, ring chunks up to 256, tile accumulators above.  With
+  // hbuf: pairs up to 64 atoms, ring chunks up to 256 (mixed), tile accumulators above.  With
   // one-sided rows chosen above 256 atoms there is no pair buffer to use: the
   // buffer holds 24 bytes per atom, not per pair, so it is withdrawn and every
   // tier evaluates in one-sided rows
@@ -153,9 +154,10 @@ cudaError_t plan_one(int max_n, int m, int64_t n_cand, int device, ljh::Plan* ou
   constexpr int threads = cta_threads_for(T);
   constexpr int TPC = threads / T;
   const size_t hist_bytes = align16(2 * (size_t)m * A * 3 * T * (MIXED ? sizeof(float) : sizeof(double)));
+  const bool buf = pair_buffer(max_n, MIXED);
   const bool on_chip =
-      !hist_global && TPC * team_smem_bytes<T>(max_n, true, hist_bytes) <= kSmemBudget;
-  const size_t smem = TPC * team_smem_bytes<T>(max_n, true, on_chip ? hist_bytes : 0);
+      !hist_global && TPC * team_smem_bytes<T>(max_n, buf, hist_bytes) <= kSmemBudget;
+  const size_t smem = TPC * team_smem_bytes<T>(max_n, buf, on_chip ? hist_bytes : 0);
   auto k = lbfgs_kernel<T, A, MIXED, POT>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
   if (e != cudaSuccess) return e;

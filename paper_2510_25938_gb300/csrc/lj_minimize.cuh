@@ -104,17 +104,15 @@ template <typename V> __device__ __forceinline__ V eps_mach();
 template <> __device__ __forceinline__ float eps_mach<float>() { return 1.1920928955078125e-7f; }
 template <> __device__ __forceinline__ double eps_mach<double>() { return 2.220446049250313e-16; }
 
-__device__ __forceinline__ float recip(float x) { return __frcp_rn(x); }
-__device__ __forceinline__ double recip(double x) { return rcp_f64(x); }
 __device__ __forceinline__ float S_sqrt(float x) { return sqrtf(x); }
 __device__ __forceinline__ double S_sqrt(double x) { return sqrt(x); }
 
 // history element (slot, atom slot a, component c) of this thread: a slot is
-// the flattened 3N vector for teams whose first warp runs the recursion (it
-// reads 16 bytes a lane), one plane per (a, c) above
-template <int T, int A>
+// the flattened 3N vector for FP32 history of teams whose first warp runs the
+// recursion (it reads 16 bytes a lane), one plane per (a, c) otherwise
+template <int T, int A, typename V>
 __device__ __forceinline__ int hidx(int slot, int a, int c, int rank) {
-  if constexpr (T <= 128) return (slot * A * T + a * T + rank) * 3 + c;
+  if constexpr (T <= 128 && sizeof(V) == 4) return (slot * A * T + a * T + rank) * 3 + c;
   else return ((slot * A + a) * 3 + c) * T + rank;
 }
 
@@ -140,6 +138,21 @@ __device__ __forceinline__ int hidx(int slot, int a, int c, int rank) {
 __device__ __forceinline__ float to_value(ff v) { return v.hi + v.lo; }
 __device__ __forceinline__ double to_value(double v) { return v; }
 
+// FP64 half pairs and row sums; V: the tier's direction type (double: the FP64 path)
+template <int T, typename V, typename Term>
+__device__ __forceinline__ void half_f64(const Team<T>& tm, int n, double* vb, Term&& term,
+                                         double gs, double* gsum, dd& e) {
+  if constexpr (sizeof(V) == 8) {
+    tri_pairs<T>(tm.rank, n, vb, term, e);
+    tm.sync();
+    tri_rows<T>(tm.rank, n, vb, gs, gsum);
+  } else {
+    half_pairs<T>(tm.rank, n, vb, term, [&](double ep) { dd_acc(e, ep); });
+    tm.sync();
+    half_rows<T>(tm.rank, n, vb, -gs, gsum);
+  }
+}
+
 // gradient of the owned atoms from the ring's sums, and this thread's g.d
 template <int T, int A, typename P, typename F, typename G>
 __device__ __forceinline__ void ring_gradient(const Team<T>& tm, int n, const F (&acc)[A][3],
@@ -160,10 +173,10 @@ __device__ __forceinline__ void pair_term_morse_f64(const PosD& a, const PosD& b
                                                     double& vz, double& e) {
   const double dx = a.x - b.x, dy = a.y - b.y, dz = a.z - b.z;
   const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
-  const double ir = rsqrt_f64(r2);
-  const double ex = exp(fma(-rr, r2 * ir, rho));
+  const double r = sqrt(r2);
+  const double ex = exp(fma(-rr, r, rho));
   e = r2 > 0.0 ? ex * (ex - 2.0) : __longlong_as_double(0x7ff0000000000000LL);
-  const double c = ex * (ex - 1.0) * ir;
+  const double c = ex * (ex - 1.0) / r;
   vx = c * dx; vy = c * dy; vz = c * dz;
 }
 
@@ -325,13 +338,10 @@ __device__ __forceinline__ void evaluate_morse(const Team<T>& tm, int n,
     double* gsum = static_cast<double*>(posv);
     const double rho = p.k.rho, rr = p.k.rho_re;
     dd e{0.0, 0.0};
-    half_pairs<T>(tm.rank, n, vb,
-                  [&](int i, int j, double& vx, double& vy, double& vz, double& ep) {
-                    pair_term_morse_f64(pos[i], pos[j], rho, rr, vx, vy, vz, ep);
-                  },
-                  [&](double ep) { dd_acc(e, ep); });   // compensated energy sum
-    tm.sync();
-    half_rows<T>(tm.rank, n, vb, -p.k.m_g, gsum);
+    auto term = [&](int i, int j, double& vx, double& vy, double& vz, double& ep) {
+      pair_term_morse_f64(pos[i], pos[j], rho, rr, vx, vy, vz, ep);
+    };
+    half_f64<T, V>(tm, n, vb, term, p.k.m_g, gsum, e);
     tm.sync();
 #pragma unroll
     for (int a = 0; a < A; ++a) {
@@ -344,7 +354,7 @@ __device__ __forceinline__ void evaluate_morse(const Team<T>& tm, int n,
       if (d) dp += (V)g[a][0] * d[a][0] + (V)g[a][1] * d[a][1] + (V)g[a][2] * d[a][2];
     }
     E = team_sum_dd<T>(tm, e) * p.k.eps;
-  } else if (T * A <= 256 && hbuf != nullptr && p.layout == LAYOUT_RING) {
+  } else if (T * A <= 256 && sizeof(V) == 4 && hbuf != nullptr && p.layout == LAYOUT_RING) {
     const PosD* pos = static_cast<const PosD*>(posv);
     const double rho = p.k.rho, rr = p.k.rho_re;
     double acc[A][3];
@@ -371,10 +381,10 @@ __device__ __forceinline__ void evaluate_morse(const Team<T>& tm, int n,
           const Q q = pos[j];
           const double dx = xi - q.x, dy = yi - q.y, dz = zi - q.z;
           const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
-          const double ir = rsqrt_f64(r2);
-          const double ex = exp(fma(-rr, r2 * ir, rho));
+          const double r = sqrt(r2);
+          const double ex = exp(fma(-rr, r, rho));
           double term = ex * (ex - 2.0);
-          double c = ex * (ex - 1.0) * ir;
+          double c = ex * (ex - 1.0) / r;
           if (j == i) {
             term = 0.0;
             c = 0.0;
@@ -460,13 +470,10 @@ __device__ __forceinline__ void evaluate(const Team<T>& tm, int n,
         double* vb = static_cast<double*>(hbuf);
         const double sig2 = p.k.sig2;
         dd e{0.0, 0.0};
-        half_pairs<T>(tm.rank, n, vb,
-                      [&](int i, int j, double& vx, double& vy, double& vz, double& ep) {
-                        pair_term_f64(pos[i], pos[j], sig2, vx, vy, vz, ep);
-                      },
-                      [&](double ep) { dd_acc(e, ep); });   // compensated energy sum
-        tm.sync();
-        half_rows<T>(tm.rank, n, vb, -p.k.gscale, gsum);
+        auto term = [&](int i, int j, double& vx, double& vy, double& vz, double& ep) {
+          pair_term_f64(pos[i], pos[j], sig2, vx, vy, vz, ep);
+        };
+        half_f64<T, V>(tm, n, vb, term, p.k.gscale, gsum, e);
         tm.sync();
         E = team_sum_dd<T>(tm, e) * p.k.e4;
       }
@@ -497,7 +504,7 @@ __device__ __forceinline__ void evaluate(const Team<T>& tm, int n,
       return;
     }
   }
-  if constexpr ((PM == 1 || std::is_same<X, double>::value) && T * A <= 256) {
+  if constexpr ((PM == 1 || std::is_same<X, double>::value) && sizeof(V) == 4 && T * A <= 256) {
     if (hbuf != nullptr && p.layout == LAYOUT_RING) {
       if constexpr (PM == 1) {
         const PosDF* pos = static_cast<const PosDF*>(posv);
@@ -768,9 +775,9 @@ __device__ __forceinline__ void warp_sum2(V& v0, V& v1) {
   }
 }
 
-// The vectors lie flat (3 N values, zeros behind them): lane l holds 16 bytes
+// FP32 vectors lie flat (3 N values, zeros behind them): lane l holds 16 bytes
 // of every 512, one vector load and at most four values a lane for LJ38 where
-// a lane with the atoms l and l + 32 had six, and while a block's products are
+// a lane with the atoms l and l + 32 had six; while a block's products are
 // being reduced its other vectors and the next block's are on their way.  1/s.y, s.y/y.y,
 // s_{t-1}.y_t and alpha are a register each, slot t's in lane t.
 // In isolation (one team, m = 10, N = 38) a direction takes 3.5k cycles: ~290 a
@@ -779,13 +786,12 @@ __device__ __forceinline__ void warp_sum2(V& v0, V& v1) {
 // launch before this form, one evaluation in the line search (run_phase) and the
 // ring order of the half pairs, 9.9 after.
 // ---------------------------------------------------------------------------
-// 16 bytes of a vector: its part of a dot product and of an update.  FP32
-// takes two values an instruction.
+// a lane's part of a vector, of a dot product and of an update: FP32 16 bytes,
+// two values an instruction; FP64 one value
 template <typename V>
 struct HistVec;
 template <>
 struct HistVec<float> {
-  static constexpr int W = 4;
   float2 a, b;
   __device__ __forceinline__ void load(const float* p) {
     const float4 q = *reinterpret_cast<const float4*>(p);
@@ -804,22 +810,12 @@ struct HistVec<float> {
 };
 template <>
 struct HistVec<double> {
-  static constexpr int W = 2;
-  double a, b;
-  __device__ __forceinline__ void load(const double* p) {
-    const double2 q = *reinterpret_cast<const double2*>(p);
-    a = q.x;
-    b = q.y;
-  }
-  __device__ __forceinline__ void store(double* p) const {
-    *reinterpret_cast<double2*>(p) = make_double2(a, b);
-  }
-  __device__ __forceinline__ void zero() { a = 0.0; b = 0.0; }
-  __device__ __forceinline__ void scale(double c) { a *= c; b *= c; }
-  __device__ __forceinline__ void add(double c, const HistVec& o) {
-    a = fma(c, o.a, a);
-    b = fma(c, o.b, b);
-  }
+  double a;
+  __device__ __forceinline__ void load(const double* p) { a = *p; }
+  __device__ __forceinline__ void store(double* p) const { *p = a; }
+  __device__ __forceinline__ void zero() { a = 0.0; }
+  __device__ __forceinline__ void scale(double c) { a *= c; }
+  __device__ __forceinline__ void add(double c, const HistVec& o) { a = fma(c, o.a, a); }
 };
 template <int NC>
 __device__ __forceinline__ float hist_dot(const HistVec<float> (&x)[NC], const HistVec<float> (&y)[NC]) {
@@ -836,12 +832,8 @@ template <int NC>
 __device__ __forceinline__ double hist_dot(const HistVec<double> (&x)[NC],
                                            const HistVec<double> (&y)[NC]) {
   double s = x[0].a * y[0].a;
-  s = fma(x[0].b, y[0].b, s);
 #pragma unroll
-  for (int c = 1; c < NC; ++c) {
-    s = fma(x[c].a, y[c].a, s);
-    s = fma(x[c].b, y[c].b, s);
-  }
+  for (int c = 1; c < NC; ++c) s = fma(x[c].a, y[c].a, s);
   return s;
 }
 
@@ -866,25 +858,28 @@ struct PairScalars<V, false> {
   __device__ __forceinline__ void set(int, int sl, V r, V g, V) { rho[sl] = r; gam[sl] = g; }
 };
 
-// the recursion of the lead warp on vectors of NC chunks of 512 bytes: q (the
-// gradient, in xb) to the direction (in xb), returns g.d
-template <int L3, int NC, typename V>
+// the recursion of the lead warp on vectors of NC parts a lane: q (the
+// gradient, in xb) to the direction (in xb), returns g.d.  FP32: chunks of 512
+// bytes of the flat vector.  FP64: the values of the atom slots (w, a) of a lane, w
+// the warp that owns them, in the order of w, a and component -- the order in
+// which the products are summed (see tri_pairs on why it matters).
+template <int T, int A, int NC, typename V>
 __device__ __forceinline__ V lead_recursion(int lane, int m, int cnt, int head,
                                             const V* __restrict__ Sh, const V* __restrict__ Yh,
                                             const PairScalars<V, true>& ps, V* xb) {
   using Vec = HistVec<V>;
-  constexpr int W = Vec::W;
+  constexpr int L3 = 3 * A * T;              // values of a slot
+  constexpr bool FLAT = sizeof(V) == 4;
+  auto at = [&](int c) {
+    return FLAT ? (c * 32 + lane) * 4 : c % (3 * A) * T + c / (3 * A) * 32 + lane;
+  };
+  auto in = [&](int c) { return !FLAT || (c + 1) * 128 <= L3 || at(c) < L3; };
   Vec q[NC], d0[NC], d1[NC], u0[NC], u1[NC];
   auto load = [&](const V* base, Vec (&o)[NC]) {
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
-      const int f = (c * 32 + lane) * W;
-      if ((c + 1) * 32 * W <= L3) {          // whole chunks
-        o[c].load(base + f);
-      } else {
-        o[c].zero();
-        if (f < L3) o[c].load(base + f);
-      }
+      if (FLAT && (c + 1) * 128 > L3) o[c].zero();   // not a whole chunk
+      if (in(c)) o[c].load(base + at(c));
     }
   };
   // slots of the pairs t (newest: cnt - 1); where there is no such pair, the
@@ -900,7 +895,7 @@ __device__ __forceinline__ V lead_recursion(int lane, int m, int cnt, int head,
   if (k0 >= m) k0 -= m;
   const V gam = ps.gam_of(k0);
   int k1 = older(k0, cnt >= 2);
-  constexpr bool kAhead = NC <= 3;           // registers for the next block's vectors
+  constexpr bool kAhead = NC * sizeof(Vec) <= 48;   // registers for the next block's vectors
   if (kAhead) {
     load(Sh + k0 * L3, d0);
     load(Sh + k1 * L3, d1);
@@ -973,9 +968,8 @@ __device__ __forceinline__ V lead_recursion(int lane, int m, int cnt, int head,
   const V dphi = -warp_sum(hist_dot(d0, q));
 #pragma unroll
   for (int c = 0; c < NC; ++c) {
-    const int f = (c * 32 + lane) * W;
     q[c].scale((V)-1);
-    if ((c + 1) * 32 * W <= L3 || f < L3) q[c].store(xb + f);
+    if (in(c)) q[c].store(xb + at(c));
   }
   return dphi;
 }
@@ -986,28 +980,31 @@ __device__ __forceinline__ V lead_two_loop(const Team<T>& tm, int n, int m, int 
                                            const PairScalars<V, true>& ps, const XG (&g)[A][3],
                                            V* xb, V (&d)[A][3]) {
   constexpr int L3 = 3 * A * T;               // values of a slot
-  constexpr int CH = 32 * HistVec<V>::W;
-  constexpr int NC = (L3 + CH - 1) / CH;
 #pragma unroll
   for (int a = 0; a < A; ++a)
 #pragma unroll
-    for (int c = 0; c < 3; ++c) xb[3 * (a * T + tm.rank) + c] = (V)g[a][c];
+    for (int c = 0; c < 3; ++c) xb[hidx<T, A, V>(0, a, c, tm.rank)] = (V)g[a][c];
   tm.sync();
   if (tm.rank < 32) {
-    // clusters that leave the last third or more of the chunks empty: fewer
-    constexpr int ND = NC > 2 ? NC * 2 / 3 : 1;
-    const V dphi = NC > 1 && 3 * n <= ND * CH
-                       ? lead_recursion<L3, ND, V>(tm.rank, m, cnt, head, Sh, Yh, ps, xb)
-                       : lead_recursion<L3, NC, V>(tm.rank, m, cnt, head, Sh, Yh, ps, xb);
-    if (NC > 1 && 3 * n <= ND * CH)           // zeros behind the chunks that were taken
-      for (int f = ND * CH + tm.rank; f < L3; f += 32) xb[f] = (V)0;
+    V dphi;
+    if constexpr (sizeof(V) == 4) {
+      // clusters that leave the last third or more of the chunks empty: fewer
+      constexpr int NC = (L3 + 127) / 128, ND = NC > 2 ? NC * 2 / 3 : 1;
+      const bool few = NC > 1 && 3 * n <= ND * 128;
+      dphi = few ? lead_recursion<T, A, ND, V>(tm.rank, m, cnt, head, Sh, Yh, ps, xb)
+                 : lead_recursion<T, A, NC, V>(tm.rank, m, cnt, head, Sh, Yh, ps, xb);
+      if (few)                                // zeros behind the chunks that were taken
+        for (int f = ND * 128 + tm.rank; f < L3; f += 32) xb[f] = (V)0;
+    } else {
+      dphi = lead_recursion<T, A, L3 / 32, V>(tm.rank, m, cnt, head, Sh, Yh, ps, xb);
+    }
     if (tm.rank == 0) xb[L3] = dphi;
   }
   tm.sync();
 #pragma unroll
   for (int a = 0; a < A; ++a)
 #pragma unroll
-    for (int c = 0; c < 3; ++c) d[a][c] = xb[3 * (a * T + tm.rank) + c];
+    for (int c = 0; c < 3; ++c) d[a][c] = xb[hidx<T, A, V>(0, a, c, tm.rank)];
   return xb[L3];
 }
 
@@ -1062,8 +1059,7 @@ __device__ __forceinline__ int run_phase(const Team<T>& tm, int n, typename P::X
       if constexpr (std::is_same<V, float>::value) {
         if (12 * A * T + 4 <= 32 * n) xb = static_cast<V*>(pos);
       } else {
-        if (hbuf != nullptr && (p.layout == LAYOUT_RING ||
-                                (p.layout == LAYOUT_HALF && 24 * A * T + 8 <= 24 * n_pairs(n))))
+        if (hbuf != nullptr && p.layout == LAYOUT_HALF && 24 * A * T + 8 <= 24 * n_pairs(n))
           xb = static_cast<V*>(hbuf);
       }
       if (cnt > 0 && xb != nullptr) {
@@ -1089,8 +1085,8 @@ __device__ __forceinline__ int run_phase(const Team<T>& tm, int n, typename P::X
         for (int a = 0; a < A; ++a)
 #pragma unroll
           for (int c = 0; c < 3; ++c) {
-            sc[a][c] = Sh[hidx<T, A>(sl, a, c, tm.rank)];
-            yc[a][c] = Yh[hidx<T, A>(sl, a, c, tm.rank)];
+            sc[a][c] = Sh[hidx<T, A, V>(sl, a, c, tm.rank)];
+            yc[a][c] = Yh[hidx<T, A, V>(sl, a, c, tm.rank)];
           }
       }
       V rho_c = ps.rho_of(slot_of(cnt - 1));
@@ -1100,8 +1096,8 @@ __device__ __forceinline__ int run_phase(const Team<T>& tm, int n, typename P::X
         for (int a = 0; a < A; ++a)
 #pragma unroll
           for (int c = 0; c < 3; ++c) {
-            sn[a][c] = Sh[hidx<T, A>(nsl, a, c, tm.rank)];
-            yn[a][c] = Yh[hidx<T, A>(nsl, a, c, tm.rank)];
+            sn[a][c] = Sh[hidx<T, A, V>(nsl, a, c, tm.rank)];
+            yn[a][c] = Yh[hidx<T, A, V>(nsl, a, c, tm.rank)];
           }
         const V rho_n = ps.rho_of(nsl);
         V part = (V)0;
@@ -1135,8 +1131,8 @@ __device__ __forceinline__ int run_phase(const Team<T>& tm, int n, typename P::X
         for (int a = 0; a < A; ++a)
 #pragma unroll
           for (int c = 0; c < 3; ++c) {
-            sn[a][c] = Sh[hidx<T, A>(nsl, a, c, tm.rank)];
-            yn[a][c] = Yh[hidx<T, A>(nsl, a, c, tm.rank)];
+            sn[a][c] = Sh[hidx<T, A, V>(nsl, a, c, tm.rank)];
+            yn[a][c] = Yh[hidx<T, A, V>(nsl, a, c, tm.rank)];
           }
         const V rho_n = ps.rho_of(nsl);
         V part = (V)0;
@@ -1355,7 +1351,7 @@ __device__ __forceinline__ int run_phase(const Team<T>& tm, int n, typename P::X
         yv[a][c] = (V)(gt[a][c] - g[a][c]);
         pr[0] += sv[a][c] * yv[a][c];
         pr[1] += yv[a][c] * yv[a][c];
-        if (prev >= 0) pr[2] += Sh[hidx<T, A>(prev, a, c, tm.rank)] * yv[a][c];
+        if (prev >= 0) pr[2] += Sh[hidx<T, A, V>(prev, a, c, tm.rank)] * yv[a][c];
       }
     // stopping-test values of the new point (||g||_inf, deadline), reduced
     // in the same pass as the curvature pair's s.y and y.y
@@ -1376,12 +1372,12 @@ __device__ __forceinline__ int run_phase(const Team<T>& tm, int n, typename P::X
       for (int a = 0; a < A; ++a)
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-          Sh[hidx<T, A>(slot, a, c, tm.rank)] = sv[a][c];
-          Yh[hidx<T, A>(slot, a, c, tm.rank)] = yv[a][c];
+          Sh[hidx<T, A, V>(slot, a, c, tm.rank)] = sv[a][c];
+          Yh[hidx<T, A, V>(slot, a, c, tm.rank)] = yv[a][c];
         }
       // 1 / s.y and the scaling s.y / y.y, formed once here instead of in every
       // recursion step; s_prev . y (undefined for the oldest pair: unused)
-      ps.set(tm.rank, slot, recip(pr[0]), pr[0] * recip(pr[1]), pr[2]);
+      ps.set(tm.rank, slot, (V)1 / pr[0], pr[0] / pr[1], pr[2]);
     }
 #pragma unroll
     for (int a = 0; a < A; ++a)

@@ -28,16 +28,24 @@ __host__ __device__ constexpr size_t align16(size_t b) { return (b + 15) & ~size
 // How FP64 and double-float evaluations take every pair once, by the largest
 // cluster of the launch, and the team's buffer for it:
 //   up to kHalfMaxN atoms    half pairs, 24 bytes per pair;
-//   up to kTileMinN          ring, 24 bytes per atom and shift of a chunk (4,096
-//                            clusters of 13..150 atoms, mixed: 17.1 ms, 19.1 with
+//   up to kTileMinN          mixed precision: ring, 24 bytes per atom and shift of a
+//                            chunk (4,096 clusters of 13..150 atoms: 17.1 ms, 19.1 with
 //                            one-sided rows, which evaluate every pair twice; 3
-//                            to 8 atom blocks leave warps idle in a tile round);
+//                            to 8 atom blocks leave warps idle in a tile round).
+//                            FP64 path: no buffer, one-sided rows -- its results hang
+//                            on the order of the sums (tri_pairs, lj_device.cuh);
+//                            a ring takes 65.6 instead of 94.4 ms (Basin Hopping, 11
+//                            walkers x 8, 5 steps, 77 atoms) but ends 8% of the
+//                            trials with another status;
 //   above                    32 x 32 tiles, 24 bytes per atom.
 constexpr int kHalfMaxN = 64;
 constexpr int kTileMinN = 256;
 enum PairLayout : int { LAYOUT_HALF = 0, LAYOUT_TILES = 1, LAYOUT_RING = 2 };
 __host__ __device__ constexpr int pair_layout(int max_n) {
   return max_n <= kHalfMaxN ? LAYOUT_HALF : max_n <= kTileMinN ? LAYOUT_RING : LAYOUT_TILES;
+}
+__host__ __device__ constexpr bool pair_buffer(int max_n, bool mixed) {
+  return mixed || pair_layout(max_n) != LAYOUT_RING;
 }
 // shifts of a ring chunk: the history of up to 256 atoms (m = 10, FP32) stays
 // on chip beside it
