@@ -29,7 +29,7 @@ struct LjConsts {
   float rho_lo;         // rho - rho_f: rho as a double-float (rho_f, rho_lo)
   float eps_f;          // eps: energy factor of a half-pair sum
   float re_f;           // re
-  float m_slope2_f;     // (rho / re) log2 e: slope of the exponent to base 2
+  float m_slope2_f, m_slope2_lo;   // (rho / re) log2 e, slope of the exponent to base 2: FP32 and its rest
 };
 
 inline LjConsts make_consts(double eps, double sigma, int pot = 0, double rho = 0.0) {
@@ -62,6 +62,7 @@ inline LjConsts make_consts(double eps, double sigma, int pot = 0, double rho = 
   k.eps_f = (float)eps;
   k.re_f = (float)sigma;
   k.m_slope2_f = (float)(k.rho_re * 1.4426950408889634074);
+  k.m_slope2_lo = (float)(k.rho_re * 1.4426950408889634074 - (double)k.m_slope2_f);
   return k;
 }
 

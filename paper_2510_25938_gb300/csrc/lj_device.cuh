@@ -336,9 +336,9 @@ __device__ __forceinline__ float ex2_approx(float x) {
 // below the distance of any 1 / a from a rounding boundary, but for the
 // significand of all ones.  Five FP64 instructions, about nine of __drcp_rn
 // (65,536 x LJ38: 2.23 ms; 2.07 without the correction, which leaves a few results
-// in a thousand an ulp off).  None on the FP64 pipe for the ends of the range: an estimate of 0 or infinity (a = 0, infinite
-// or so small that its inverse overflows) is returned as it is, chosen by its
-// exponent bits on the integer pipe.
+// in a thousand an ulp off).  None on the FP64 pipe for the ends of the range: an
+// estimate of 0 or infinity (a = 0, infinite or so small that its inverse overflows)
+// is returned as it is, chosen by its exponent bits on the integer pipe.
 __device__ __forceinline__ bool f64_end(double r) {   // 0, subnormal, infinite or NaN
   const int ex = __double2hiint(r) & 0x7ff00000;
   return ex == 0 || ex == 0x7ff00000;
@@ -349,14 +349,6 @@ __device__ __forceinline__ double rcp_f64(double a, double one = 1.0) {
   const double e = fma(-a, r, one);
   double y = fma(r, fma(e, e, e), r);
   y = fma(y, fma(-a, y, one), y);
-  return f64_end(r) ? r : y;
-}
-// 1 / sqrt(a) in FP64, likewise: with e = 1 - a r^2, r (1 + e/2 + 3 e^2 / 8)
-__device__ __forceinline__ double rsqrt_f64(double a) {
-  double r;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
-  const double e = fma(-(a * r), r, 1.0);
-  const double y = fma(r * e, fma(0.375, e, 0.5), r);
   return f64_end(r) ? r : y;
 }
 

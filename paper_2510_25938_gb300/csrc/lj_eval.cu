@@ -30,8 +30,8 @@ __global__ void __launch_bounds__(256, 2) eval_ring_f32_kernel(ljh::EvalArgs a, 
   const bool parts_buf = MULTI && (pl.P > 1 || S > 1);
   ff* es = reinterpret_cast<ff*>(own + (parts_buf ? B : 0));
   ff* ecl = reinterpret_cast<ff*>(reinterpret_cast<unsigned char*>(es) + (size_t)B * 16);
-  const float k0 = POT == LJ_POT_LJ ? a.k.sig2_f : -a.k.re_f;
-  const float k1 = POT == LJ_POT_LJ ? 0.f : -a.k.m_slope2_f;
+  const RingK k = POT == LJ_POT_LJ ? RingK{a.k.sig2_f, 0.f, 0.f}
+                                   : RingK{-a.k.re_f, -a.k.m_slope2_f, -a.k.m_slope2_lo};
   const float gs = POT == LJ_POT_LJ ? a.k.gscale_f : a.k.m_g_f;
   const double ef = POT == LJ_POT_LJ ? a.k.e4 : a.k.eps;
   const IO* __restrict__ xin = static_cast<const IO*>(a.x);
@@ -108,17 +108,17 @@ __global__ void __launch_bounds__(256, 2) eval_ring_f32_kernel(ljh::EvalArgs a, 
     const int GP = MULTI ? S * P : 1, gp = MULTI ? srank * P + p : 0;
     // the pairs inside the groups go to the last part, which has no more
     // shifts than any other
-    if (live && gp == GP - 1) intra<G, POT, SIG>(N, pos[pslot + g], k0, k1, o, e);
+    if (live && gp == GP - 1) intra<G, POT, SIG>(N, pos[pslot + g], k, o, e);
     const bool even = (NG & 1) == 0;
     for (int kc = 0; kc * GP < H || kc == 0; kc += KS) {
       if (kc > 0) __syncthreads();           // the last chunk's readers are done
       if (live) {
         for (int s = 0; s < KS; ++s) {
-          const int k = 1 + (kc + s) * GP + gp;
-          if (k > H) break;
-          int t = g + k;
+          const int sh = 1 + (kc + s) * GP + gp;
+          if (sh > H) break;
+          int t = g + sh;
           if (t >= NG) t -= NG;
-          shift<G, POT, SIG>(N, pos[pslot + t], even && k == H, g < H, k0, k1, o, e,
+          shift<G, POT, SIG>(N, pos[pslot + t], even && sh == H, g < H, k, o, e,
                              react[s * B + slot + t]);
         }
         if (!UNEVEN) es[tid] = e;

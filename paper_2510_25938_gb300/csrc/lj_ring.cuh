@@ -100,19 +100,27 @@ __device__ __forceinline__ void v2_add(V2& a, const V2& b) {
   a.x = __fadd2_rn(a.x, b.x); a.y = __fadd2_rn(a.y, b.y); a.z = __fadd2_rn(a.z, b.z);
 }
 
+// constants of a pair term.  Eq. (1): a = sigma^2.  Morse: a = -re and b + c =
+// -(rho / re) log2 e, b its FP32 rounding
+struct RingK {
+  float a, b, c;
+};
+
 // One packed operation: the two pairs (X.lane0, Y.lane0) and (X.lane1,
 // Y.lane1), given NX = -X (negation is exact, so y + (-x) rounds like y - x):
 // d = y - x, the factor c of the force term c d on x (in units of the
 // potential's gradient factor, sign of sum_j c (x_j - x_i); its reaction on y
 // is subtracted), and eb += e.
-// Eq. (1): s2 = sigma^2 / r^2 (k0 = sigma^2 where SIG), c = s2 s6 (2 s6 - 1),
-// e = s6 (s6 - 1).  Morse: with k0 = -re, k1 = -(rho / re) log2 e the
-// exponential is 2^(k1 (r + k0)); r + k0 is one FMA from r^2 and 1 / r, so it
-// carries no rounding of r itself; c = m (m - 1) / r, e = m (m - 2).
+// Eq. (1): s2 = sigma^2 / r^2, c = s2 s6 (2 s6 - 1), e = s6 (s6 - 1).
+// Morse: the exponential is 2^((b + c)(r - re)); r - re is one FMA from r^2 and
+// 1 / r, so it carries no rounding of r itself.  The slope takes two words: its
+// rounding is the same for every pair and would not average out (rho = 6: energies
+// of 500 atoms off by 2.4e-8, 0.75e-8 before the ring layout); c = m (m - 1) / r,
+// e = m (m - 2).
 // With the force and the reaction 19 FP32 lane operations a pair and one
-// (Morse: two) on the MUFU.
+// (Morse: 20 and two) on the MUFU.
 template <int POT, bool SIG>
-__device__ __forceinline__ void ring_op(const V2& NX, const V2& Y, float k0, float k1, V2& d,
+__device__ __forceinline__ void ring_op(const V2& NX, const V2& Y, const RingK& k, V2& d,
                                         float2& c, float2& eb) {
   d.x = __fadd2_rn(Y.x, NX.x);
   d.y = __fadd2_rn(Y.y, NX.y);
@@ -120,14 +128,15 @@ __device__ __forceinline__ void ring_op(const V2& NX, const V2& Y, float k0, flo
   const float2 r2 = __ffma2_rn(d.x, d.x, __ffma2_rn(d.y, d.y, __fmul2_rn(d.z, d.z)));
   if constexpr (POT == LJ_POT_LJ) {
     float2 s2 = make_float2(rcp_approx(r2.x), rcp_approx(r2.y));
-    if constexpr (SIG) s2 = __fmul2_rn(s2, f2(k0));
+    if constexpr (SIG) s2 = __fmul2_rn(s2, f2(k.a));
     const float2 s6 = __fmul2_rn(__fmul2_rn(s2, s2), s2);
     const float2 t = __fadd2_rn(s6, f2(-1.f));
     eb = __ffma2_rn(s6, t, eb);
     c = __fmul2_rn(__fmul2_rn(s2, s6), __fadd2_rn(s6, t));
   } else {
     const float2 ir = make_float2(rsqrt_approx(r2.x), rsqrt_approx(r2.y));
-    const float2 x = __fmul2_rn(__ffma2_rn(r2, ir, f2(k0)), f2(k1));
+    const float2 u = __ffma2_rn(r2, ir, f2(k.a));
+    const float2 x = __ffma2_rn(u, f2(k.b), __fmul2_rn(u, f2(k.c)));
     const float2 m = make_float2(ex2_approx(x.x), ex2_approx(x.y));
     eb = __ffma2_rn(m, __fadd2_rn(m, f2(-2.f)), eb);
     c = __fmul2_rn(__fmul2_rn(m, __fadd2_rn(m, f2(-1.f))), ir);
@@ -273,7 +282,7 @@ __device__ __forceinline__ V2 partner(const PosRing<G>& rb, int j, const float4&
 // the pairs inside a group: operand h with the atoms above 2h + 1 (from the own
 // record), and the pairs (2h, 2h + 1) of two operands at a time
 template <int G, int POT, bool SIG>
-__device__ __forceinline__ void intra(const V2 (&N)[G / 2], const PosRing<G>& own, float k0, float k1,
+__device__ __forceinline__ void intra(const V2 (&N)[G / 2], const PosRing<G>& own, const RingK& k,
                                       Own<G>& o, ff& e) {
   float2 eb = f2(0.f);
 #pragma unroll
@@ -284,7 +293,7 @@ __device__ __forceinline__ void intra(const V2 (&N)[G / 2], const PosRing<G>& ow
     for (int h = 0; h < j / 2; ++h) {
       V2 d;
       float2 c;
-      ring_op<POT, SIG>(N[h], b, k0, k1, d, c, eb);
+      ring_op<POT, SIG>(N[h], b, k, d, c, eb);
       if (h == 0) r = v2_scale(c, d);
       else v2_fma(r, c, d);
       v2_fma(o.f[h], c, d);
@@ -305,7 +314,7 @@ __device__ __forceinline__ void intra(const V2 (&N)[G / 2], const PosRing<G>& ow
                          make_float2(A.z.x, B.z.x)},
                       V2{make_float2(-A.x.y, -B.x.y), make_float2(-A.y.y, -B.y.y),
                          make_float2(-A.z.y, -B.z.y)},
-                      k0, k1, d, c, eb);
+                      k, d, c, eb);
     const V2 r = v2_scale(c, d);
     v2_add(o.f[h], V2{make_float2(r.x.x, -r.x.x), make_float2(r.y.x, -r.y.x),
                       make_float2(r.z.x, -r.z.x)});
@@ -320,7 +329,7 @@ __device__ __forceinline__ void intra(const V2 (&N)[G / 2], const PosRing<G>& ow
 // are summed in FP32 over 16 pairs a lane at most, then in float-float.
 template <int G, int POT, bool SIG>
 __device__ __forceinline__ void shift(const V2 (&N)[G / 2], const PosRing<G>& rb, bool split,
-                                      bool lower, float k0, float k1, Own<G>& o, ff& e,
+                                      bool lower, const RingK& k, Own<G>& o, ff& e,
                                       SlotF<G>& w) {
   float px[4], py[4], pz[4];               // reactions on four of the partner's atoms
   auto fold = [&](int j, const V2& r) {
@@ -345,7 +354,7 @@ __device__ __forceinline__ void shift(const V2 (&N)[G / 2], const PosRing<G>& rb
       for (int h = 0; h < G / 2; ++h) {
         V2 d;
         float2 c;
-        ring_op<POT, SIG>(N[h], b, k0, k1, d, c, eb);
+        ring_op<POT, SIG>(N[h], b, k, d, c, eb);
         if (h == 0) r = v2_scale(c, d);
         else v2_fma(r, c, d);
         v2_fma(o.f[h], c, d);
@@ -368,7 +377,7 @@ __device__ __forceinline__ void shift(const V2 (&N)[G / 2], const PosRing<G>& rb
       const V2 b = partner(rb, j, zz);
       V2 d;
       float2 c;
-      ring_op<POT, SIG>(lower || !(u & 1) ? N[0] : N[1], b, k0, k1, d, c, eb);
+      ring_op<POT, SIG>(lower || !(u & 1) ? N[0] : N[1], b, k, d, c, eb);
       r[u] = v2_scale(c, d);
     }
     v2_add(o.f[0], r[0]);
@@ -412,7 +421,7 @@ __device__ __forceinline__ void shift(const V2 (&N)[G / 2], const PosRing<G>& rb
           if (lower && h >= G / 4) continue;
           V2 d;
           float2 c;
-          ring_op<POT, SIG>(N[h], b, k0, k1, d, c, eb);
+          ring_op<POT, SIG>(N[h], b, k, d, c, eb);
           v2_fma(r, c, d);
           v2_fma(o.f[h], c, d);
         }
@@ -449,11 +458,13 @@ __device__ __forceinline__ void ringd_op(double ax, double ay, double az, double
     e = fma(s6, t, e);
     c = (s2 * s6) * (s6 + t);
   } else {
-    const double ir = rsqrt_f64(r2);
-    const double m = exp(fma(-k1, r2 * ir, k0));
+    // an ulp of r is rho ulps of m: r is the correctly rounded root.  A reciprocal
+    // root within an ulp for both r and 1 / r made gradients 1.5 times less exact
+    const double r = sqrt(r2);
+    const double m = exp(fma(-k1, r, k0));
     const double term = m * (m - 2.0);
     e += r2 > 0.0 ? term : __longlong_as_double(0x7ff0000000000000LL);
-    c = m * (m - 1.0) * ir;
+    c = m * (m - 1.0) / r;
   }
   fx = fma(c, dx, fx); fy = fma(c, dy, fy); fz = fma(c, dz, fz);
   px = fma(c, dx, px); py = fma(c, dy, py); pz = fma(c, dz, pz);
