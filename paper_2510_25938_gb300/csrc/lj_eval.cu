@@ -102,9 +102,10 @@ __global__ void __launch_bounds__(256, 2) eval_ring_f32_kernel(ljh::EvalArgs a, 
         N[h] = V2{make_float2(-q[6 * h], -q[6 * h + 3]), make_float2(-q[6 * h + 1], -q[6 * h + 4]),
                   make_float2(-q[6 * h + 2], -q[6 * h + 5])};
     }
-    ff e{0.f, 0.f};
-    Own<G> o;
+    E2 e{f2(0.f), f2(0.f)};
+    Own<G> o, tot;
     own_zero(o);
+    own_zero(tot);
     const int GP = MULTI ? S * P : 1, gp = MULTI ? srank * P + p : 0;
     // the pairs inside the groups go to the last part, which has no more
     // shifts than any other
@@ -121,24 +122,34 @@ __global__ void __launch_bounds__(256, 2) eval_ring_f32_kernel(ljh::EvalArgs a, 
           shift<G, POT, SIG>(N, pos[pslot + t], even && sh == H, g < H, k, o, e,
                              react[s * B + slot + t]);
         }
-        if (!UNEVEN) es[tid] = e;
+        if (!UNEVEN) es[tid] = e2_total(e);
       }
       // zeros from a candidate's idle threads, NaN for a bad size
-      if (UNEVEN && here) es[tid] = bad && g == 0 ? ff{__int_as_float(0x7fc00000), 0.f} : e;
+      if (UNEVEN && here) es[tid] = bad && g == 0 ? ff{__int_as_float(0x7fc00000), 0.f} : e2_total(e);
       __syncthreads();
+      // forces are summed in parts -- the reactions by themselves, then (several
+      // chunks) chunk by chunk -- and not in one FP32 sum over all atoms, whose error
+      // grows with their number (1,024 x 500 atoms: 5.5e-7 of the gradient so, 4.2e-7 in
+      // parts; 111 and 115 us with the energies' blocks)
       if (live && (MULTI || gout)) {
+        Own<G> r;
+        own_zero(r);
         for (int s = 0; s < KS; ++s) {
           if (1 + (kc + s) * GP + gp > H) break;
-          own_slot<false>(o, react[s * B + slot + g]);
+          own_slot(r, react[s * B + slot + g]);
         }
+        own_add<false>(o, r);
       }
       if (!MULTI) break;
+      own_add<true>(tot, o);
+      own_zero(o);
     }
+    if (MULTI) o = tot;
     if (MULTI && P > 1) {                    // parts in the order of p
       if (live && p > 0) own_write(o, own[slot + g]);
       __syncthreads();
       if (live && p == 0)
-        for (int pp = 1; pp < P; ++pp) own_slot<true>(o, own[slot + pp * NG + g]);
+        for (int pp = 1; pp < P; ++pp) own_slot(o, own[slot + pp * NG + g]);
     }
     if (tid < 32)
       sum_energies(es, pl.C, UNEVEN ? NS : NG * P, [&](int c, ff s) {
@@ -151,7 +162,7 @@ __global__ void __launch_bounds__(256, 2) eval_ring_f32_kernel(ljh::EvalArgs a, 
       cl.sync();
       own_zero(o);
       if (live && p == 0 && g % S == srank)
-        for (int s = 0; s < S; ++s) own_slot<true>(o, *cl.map_shared_rank(&own[slot + g], s));
+        for (int s = 0; s < S; ++s) own_slot(o, *cl.map_shared_rank(&own[slot + g], s));
       if (srank == 0 && tid < pl.C && c0 + tid < a.n_cand) {
         ff s = ecl[tid];
         for (int r = 1; r < S; ++r) acc_pair(s, *cl.map_shared_rank(&ecl[tid], r));
@@ -235,9 +246,8 @@ __global__ void __launch_bounds__(256, POT == LJ_POT_LJ ? 2 : 1) eval_ring_f64_k
       for (int j = 0; j < G; ++j) { q.x[j] = r.x[j]; q.y[j] = r.y[j]; q.z[j] = r.z[j]; }
     }
     dd e{0.0, 0.0};
-    double eb = 0.0;
     const int GP = S * P, gp = srank * P + p;
-    if (live && gp == GP - 1) intra_d<G, POT, SIG>(q, one, k0, k1, f, eb);
+    if (live && gp == GP - 1) intra_d<G, POT, SIG>(q, one, k0, k1, f, e);
     const bool even = (NG & 1) == 0;
     for (int kc = 0; kc * GP < H || kc == 0; kc += KS) {
       if (kc > 0) __syncthreads();
@@ -247,15 +257,9 @@ __global__ void __launch_bounds__(256, POT == LJ_POT_LJ ? 2 : 1) eval_ring_f64_k
           if (k > H) break;
           int t = g + k;
           if (t >= NG) t -= NG;
-          shift_d<G, POT, SIG>(q, pos[pslot + t], even && k == H, g < H, one, k0, k1, f, eb,
+          shift_d<G, POT, SIG>(q, pos[pslot + t], even && k == H, g < H, one, k0, k1, f, e,
                                react[s * B + slot + t]);
-          if ((s + 1) * G * G % 16 < G * G) {   // ~16 pairs in FP64, then double-double
-            acc_pair(e, dd{eb, 0.0});
-            eb = 0.0;
-          }
         }
-        if (eb != 0.0) acc_pair(e, dd{eb, 0.0});
-        eb = 0.0;
         es[tid] = e;
       }
       __syncthreads();
@@ -442,8 +446,11 @@ RingLaunch ring_plan(const ljh::EvalArgs& a, int sms) {
 template <typename K>
 cudaError_t launch_ring(K k, const ljh::EvalArgs& a, const RingLaunch& r, cudaStream_t s) {
   const size_t smem = ring_smem(r.B, r.pl, a.prec != LJ_PREC_FP64, r.G);
+  // The limit belongs to the kernel and not to the launch, and one kernel serves many
+  // shapes (53 KB for 1,024 x 500 atoms, 107 KB for 256 x 1,024): it is always
+  // the most there is, so that no thread lowers it between another's two calls.
   if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
     if (e != cudaSuccess) return e;
   }
   const long long need = (a.n_cand + r.pl.C - 1) / r.pl.C;

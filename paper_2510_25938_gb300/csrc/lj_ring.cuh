@@ -94,6 +94,29 @@ __device__ __forceinline__ void sum_energies(const E* es, int C, int cnt, F&& st
 struct V2 {
   float2 x, y, z;
 };
+
+// a thread's energy: in each of the two lanes a running double-float sum (Sum2, as
+// df_acc).  Seven packed operations a block of terms, and the lanes stay apart
+// to the end: adding them first, in FP32, took nine scalar ones and was the largest
+// rounding of a block (65,536 x LJ38: energies off by 6.19e-8 in 57.4 us, 6.06e-8 in
+// 59.4 so; 6.08e-8 with blocks of eight pairs in the first ring kernel, 65.5 us).
+struct E2 {
+  float2 hi, lo;
+};
+__device__ __forceinline__ float2 sub2(const float2& a, const float2& b) {
+  return __ffma2_rn(b, f2(-1.f), a);       // exact product: one rounding
+}
+__device__ __forceinline__ void e2_acc(E2& e, const float2& v) {
+  const float2 s = __fadd2_rn(e.hi, v);
+  const float2 bb = sub2(s, e.hi);
+  const float2 err = __fadd2_rn(sub2(e.hi, sub2(s, bb)), sub2(v, bb));
+  e.hi = s;
+  e.lo = __fadd2_rn(e.lo, err);
+}
+__device__ __forceinline__ ff e2_total(const E2& e) {
+  const ff t = ff_two_sum(e.hi.x, e.hi.y);
+  return ff{t.hi, __fadd_rn(t.lo, __fadd_rn(e.lo.x, e.lo.y))};
+}
 __device__ __forceinline__ V2 v2_zero() { return V2{f2(0.f), f2(0.f), f2(0.f)}; }
 __device__ __forceinline__ V2 v2_dup(float x, float y, float z) { return V2{f2(x), f2(y), f2(z)}; }
 __device__ __forceinline__ void v2_add(V2& a, const V2& b) {
@@ -223,15 +246,20 @@ __device__ __forceinline__ void own_zero(Own<G>& o) {
   for (int h = 0; h < G / 2; ++h) o.f[h] = v2_zero();
 }
 template <bool ADD, int G>
+__device__ __forceinline__ void own_add(Own<G>& o, const Own<G>& r) {
+  // f + s r by one FMA: exact product
+#pragma unroll
+  for (int h = 0; h < G / 2; ++h) v2_fma(o.f[h], f2(ADD ? 1.f : -1.f), r.f[h]);
+}
+template <int G>
 __device__ __forceinline__ void own_slot(Own<G>& o, const SlotF<G>& r) {
-  const float2 s = f2(ADD ? 1.f : -1.f);   // f + s r by one FMA: exact product
 #pragma unroll
   for (int v = 0; v < G / 4; ++v) {
     const float4 x = reinterpret_cast<const float4*>(r.x)[v];
     const float4 y = reinterpret_cast<const float4*>(r.y)[v];
     const float4 z = reinterpret_cast<const float4*>(r.z)[v];
-    v2_fma(o.f[2 * v], s, V2{make_float2(x.x, x.y), make_float2(y.x, y.y), make_float2(z.x, z.y)});
-    v2_fma(o.f[2 * v + 1], s,
+    v2_add(o.f[2 * v], V2{make_float2(x.x, x.y), make_float2(y.x, y.y), make_float2(z.x, z.y)});
+    v2_add(o.f[2 * v + 1],
            V2{make_float2(x.z, x.w), make_float2(y.z, y.w), make_float2(z.z, z.w)});
   }
 }
@@ -283,8 +311,8 @@ __device__ __forceinline__ V2 partner(const PosRing<G>& rb, int j, const float4&
 // record), and the pairs (2h, 2h + 1) of two operands at a time
 template <int G, int POT, bool SIG>
 __device__ __forceinline__ void intra(const V2 (&N)[G / 2], const PosRing<G>& own, const RingK& k,
-                                      Own<G>& o, ff& e) {
-  float2 eb = f2(0.f);
+                                      Own<G>& o, E2& e) {
+  float2 eb[2] = {f2(0.f), f2(0.f)};
 #pragma unroll
   for (int j = 2; j < G; ++j) {
     const V2 b = partner(own, j, own.zz[j / 2]);
@@ -293,7 +321,7 @@ __device__ __forceinline__ void intra(const V2 (&N)[G / 2], const PosRing<G>& ow
     for (int h = 0; h < j / 2; ++h) {
       V2 d;
       float2 c;
-      ring_op<POT, SIG>(N[h], b, k, d, c, eb);
+      ring_op<POT, SIG>(N[h], b, k, d, c, eb[G > 4 ? j & 1 : 0]);
       if (h == 0) r = v2_scale(c, d);
       else v2_fma(r, c, d);
       v2_fma(o.f[h], c, d);
@@ -314,22 +342,23 @@ __device__ __forceinline__ void intra(const V2 (&N)[G / 2], const PosRing<G>& ow
                          make_float2(A.z.x, B.z.x)},
                       V2{make_float2(-A.x.y, -B.x.y), make_float2(-A.y.y, -B.y.y),
                          make_float2(-A.z.y, -B.z.y)},
-                      k, d, c, eb);
+                      k, d, c, eb[G > 4 ? h / 2 & 1 : 0]);
     const V2 r = v2_scale(c, d);
     v2_add(o.f[h], V2{make_float2(r.x.x, -r.x.x), make_float2(r.y.x, -r.y.x),
                       make_float2(r.z.x, -r.z.x)});
     v2_add(o.f[h + 1], V2{make_float2(r.x.y, -r.x.y), make_float2(r.y.y, -r.y.y),
                           make_float2(r.z.y, -r.z.y)});
   }
-  df_acc(e, ff{__fadd_rn(eb.x, eb.y), 0.f});
+  e2_acc(e, G > 4 ? __fadd2_rn(eb[0], eb[1]) : eb[0]);
 }
 
 // one shift: the G^2 pairs (a split shift: half of them) of the own group,
 // negated in N, with the partner's record; its reaction goes to w.  Energies
-// are summed in FP32 over 16 pairs a lane at most, then in float-float.
+// are summed in FP32 over four (G = 8: eight) pairs a lane, two such sums at a
+// time, then in double-float.
 template <int G, int POT, bool SIG>
 __device__ __forceinline__ void shift(const V2 (&N)[G / 2], const PosRing<G>& rb, bool split,
-                                      bool lower, const RingK& k, Own<G>& o, ff& e,
+                                      bool lower, const RingK& k, Own<G>& o, E2& e,
                                       SlotF<G>& w) {
   float px[4], py[4], pz[4];               // reactions on four of the partner's atoms
   auto fold = [&](int j, const V2& r) {
@@ -344,7 +373,7 @@ __device__ __forceinline__ void shift(const V2 (&N)[G / 2], const PosRing<G>& rb
   };
   if (!split) {
     float4 zz;
-    float2 eb = f2(0.f);
+    float2 eb[2] = {f2(0.f), f2(0.f)};
 #pragma unroll
     for (int j = 0; j < G; ++j) {
       if (!(j & 1)) zz = rb.zz[j / 2];
@@ -354,7 +383,7 @@ __device__ __forceinline__ void shift(const V2 (&N)[G / 2], const PosRing<G>& rb
       for (int h = 0; h < G / 2; ++h) {
         V2 d;
         float2 c;
-        ring_op<POT, SIG>(N[h], b, k, d, c, eb);
+        ring_op<POT, SIG>(N[h], b, k, d, c, eb[h & 1]);
         if (h == 0) r = v2_scale(c, d);
         else v2_fma(r, c, d);
         v2_fma(o.f[h], c, d);
@@ -362,8 +391,8 @@ __device__ __forceinline__ void shift(const V2 (&N)[G / 2], const PosRing<G>& rb
       fold(j, r);
       if ((j & 3) == 3) {
         put(j / 4);
-        df_acc(e, ff{__fadd_rn(eb.x, eb.y), 0.f});
-        eb = f2(0.f);
+        e2_acc(e, __fadd2_rn(eb[0], eb[1]));
+        eb[0] = eb[1] = f2(0.f);
       }
     }
   } else if constexpr (G == 4) {
@@ -398,7 +427,7 @@ __device__ __forceinline__ void shift(const V2 (&N)[G / 2], const PosRing<G>& rb
       fold(3, r[2]);
     }
     put(0);
-    df_acc(e, ff{__fadd_rn(eb.x, eb.y), 0.f});
+    e2_acc(e, eb);
   } else {
     // lower thread the lower half of its atoms with all of b, upper thread all
     // of its atoms with the upper half of b
@@ -411,7 +440,7 @@ __device__ __forceinline__ void shift(const V2 (&N)[G / 2], const PosRing<G>& rb
     }
 #pragma unroll 1
     for (int j = j0; j < G; j += 4) {
-      float2 eb = f2(0.f);
+      float2 eb[2] = {f2(0.f), f2(0.f)};
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const V2 b = partner(rb, j + u, rb.zz[(j + u) / 2]);
@@ -421,14 +450,14 @@ __device__ __forceinline__ void shift(const V2 (&N)[G / 2], const PosRing<G>& rb
           if (lower && h >= G / 4) continue;
           V2 d;
           float2 c;
-          ring_op<POT, SIG>(N[h], b, k, d, c, eb);
+          ring_op<POT, SIG>(N[h], b, k, d, c, eb[h & 1]);
           v2_fma(r, c, d);
           v2_fma(o.f[h], c, d);
         }
         fold(u, r);
       }
       put(j / 4);
-      df_acc(e, ff{__fadd_rn(eb.x, eb.y), 0.f});
+      e2_acc(e, __fadd2_rn(eb[0], eb[1]));
     }
   }
 }
@@ -494,9 +523,20 @@ __device__ __forceinline__ void load_group_d(const IO* __restrict__ x, int n, in
   }
 }
 
+// Energies: four pairs at most in FP64, then double-double; Morse, whose exponential
+// makes the rest cheap, pair by pair.
+template <int POT>
+__device__ __forceinline__ void fold_d(dd& e, double& eb, bool block) {
+  if (POT != LJ_POT_LJ || block) {
+    dd_acc(e, eb);
+    eb = 0.0;
+  }
+}
+
 template <int G, int POT, bool SIG>
 __device__ __forceinline__ void intra_d(const GroupD<G>& q, double one, double k0, double k1,
-                                        GroupD<G>& f, double& eb) {
+                                        GroupD<G>& f, dd& e) {
+  double eb = 0.0;
 #pragma unroll
   for (int i = 0; i < G; ++i)
 #pragma unroll
@@ -504,6 +544,7 @@ __device__ __forceinline__ void intra_d(const GroupD<G>& q, double one, double k
       double px = 0, py = 0, pz = 0;
       ringd_op<POT, SIG>(q.x[i], q.y[i], q.z[i], q.x[j], q.y[j], q.z[j], one, k0, k1, f.x[i],
                          f.y[i], f.z[i], px, py, pz, eb);
+      fold_d<POT>(e, eb, j == G - 1 && (G > 3 && i == 0 || i == G - 2));
       f.x[j] -= px; f.y[j] -= py; f.z[j] -= pz;
     }
 }
@@ -511,16 +552,19 @@ __device__ __forceinline__ void intra_d(const GroupD<G>& q, double one, double k
 template <int G, int POT, bool SIG>
 __device__ __forceinline__ void shift_d(const GroupD<G>& q, const PosDG<G>& rb, bool split,
                                         bool lower, double one, double k0, double k1, GroupD<G>& f,
-                                        double& eb, PosDG<G>& w) {
+                                        dd& e, PosDG<G>& w) {
   GroupD<G> p;
   group_zero(p);
+  double eb = 0.0;
   if (!split) {
 #pragma unroll
     for (int j = 0; j < G; ++j)
 #pragma unroll
-      for (int i = 0; i < G; ++i)
+      for (int i = 0; i < G; ++i) {
         ringd_op<POT, SIG>(q.x[i], q.y[i], q.z[i], rb.x[j], rb.y[j], rb.z[j], one, k0, k1, f.x[i],
                            f.y[i], f.z[i], p.x[j], p.y[j], p.z[j], eb);
+        fold_d<POT>(e, eb, i == G - 1 && (G > 2 || j == G - 1));
+      }
   } else {
     // lower thread the lower half of its atoms with all of b, upper thread
     // all of its atoms with the upper half of b
@@ -528,9 +572,11 @@ __device__ __forceinline__ void shift_d(const GroupD<G>& q, const PosDG<G>& rb, 
     for (int j = 0; j < G; ++j)
 #pragma unroll
       for (int i = 0; i < G; ++i)
-        if (lower ? i < G / 2 : j >= G / 2)
+        if (lower ? i < G / 2 : j >= G / 2) {
           ringd_op<POT, SIG>(q.x[i], q.y[i], q.z[i], rb.x[j], rb.y[j], rb.z[j], one, k0, k1,
                              f.x[i], f.y[i], f.z[i], p.x[j], p.y[j], p.z[j], eb);
+          fold_d<POT>(e, eb, i == (lower ? G / 2 : G) - 1 && (G > 2 || j == G - 1));
+        }
   }
 #pragma unroll
   for (int j = 0; j < G; ++j) { w.x[j] = p.x[j]; w.y[j] = p.y[j]; w.z[j] = p.z[j]; }
