@@ -144,13 +144,13 @@ __device__ __forceinline__ void df_acc(ff& s, ff v) {
 template <int T>
 __device__ __forceinline__ ff team_sum_ff(const Team<T>& tm, ff v) {
   // both partners of a butterfly step form the same sums: TwoSum's results
-  // and (v.lo + w.lo) do not depend on the order of the operands
+  // and (v.lo + w.lo) do not depend on the order of the operands.  Every step
+  // renormalises: the threads' low words, gathered over hundreds of pairs, are
+  // far above an ulp of the high ones, and plain FP32 sums of them round by
+  // about as much as the line search resolves (Morse, 400 atoms: 9 of 1,500
+  // quenches failed their last line search).
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const ff w{shfl_xor(v.hi, o), shfl_xor(v.lo, o)};
-    const ff t = ff_two_sum(v.hi, w.hi);
-    v = ff{t.hi, __fadd_rn(t.lo, __fadd_rn(v.lo, w.lo))};
-  }
+  for (int o = 16; o > 0; o >>= 1) v = ff_add(v, ff{shfl_xor(v.hi, o), shfl_xor(v.lo, o)});
   if constexpr (T > 32) {
     constexpr int NW = T / 32;
     float* buf = reinterpret_cast<float*>(tm.scratch());
@@ -161,7 +161,7 @@ __device__ __forceinline__ ff team_sum_ff(const Team<T>& tm, ff v) {
     tm.sync();
     ff s{buf[0], buf[1]};
 #pragma unroll
-    for (int w = 1; w < NW; ++w) df_acc(s, ff{buf[2 * w], buf[2 * w + 1]});
+    for (int w = 1; w < NW; ++w) s = ff_add(s, ff{buf[2 * w], buf[2 * w + 1]});
     v = s;
   }
   return v;
@@ -245,8 +245,7 @@ __device__ __forceinline__ void team_sum_ff_f(const Team<T>& tm, ff& e, float& x
   for (int o = 16; o > 0; o >>= 1) {
     const ff w{shfl_xor(e.hi, o), shfl_xor(e.lo, o)};
     x += shfl_xor(x, o);
-    const ff t = ff_two_sum(e.hi, w.hi);
-    e = ff{t.hi, __fadd_rn(t.lo, __fadd_rn(e.lo, w.lo))};
+    e = ff_add(e, w);
   }
   if constexpr (T > 32) {
     constexpr int NW = T / 32;
@@ -261,7 +260,7 @@ __device__ __forceinline__ void team_sum_ff_f(const Team<T>& tm, ff& e, float& x
     float t = buf[2];
 #pragma unroll
     for (int w = 1; w < NW; ++w) {
-      df_acc(s, ff{buf[3 * w], buf[3 * w + 1]});
+      s = ff_add(s, ff{buf[3 * w], buf[3 * w + 1]});
       t += buf[3 * w + 2];
     }
     e = s;
