@@ -54,6 +54,8 @@ struct LbfgsArgs {
   int hist_on_chip;            // history in shared memory (hist unused)
   const int* list = nullptr;   // bucketed launch: candidate indices of this bucket
   const unsigned* list_count = nullptr;   // ... and their number (device)
+  unsigned count_min = 0, count_max = ~0u;   // ... for which this launch is meant: above
+                                             // count_min, up to count_max
 };
 
 // size classes of a bucketed uneven batch (upper atom count per bucket)
@@ -91,6 +93,8 @@ struct Plan {
   size_t slot_bytes; // bytes per history slot
   int cluster = 1;   // CTAs per thread-block cluster (Basin Hopping: K)
   int hist_on_chip = 0;   // L-BFGS history in shared memory
+  int many = 0;           // L-BFGS shapes with two builds: the one for more than this many
+                          // candidates is meant (0: the other, or there is only one)
 };
 
 // largest atom count this build supports

@@ -5,6 +5,8 @@
 // different iteration counts; the queue keeps every team busy until the
 // batch is drained.
 #pragma once
+#include <algorithm>
+
 #include "lj_internal.h"
 #include "lj_minimize.cuh"
 #include "lj_teams.cuh"
@@ -30,19 +32,27 @@ __device__ __forceinline__ MinParams to_dev(const ljh::MinParamsH& h) {
 // (4,096 x LJ38: 2.64 against 2.82 ms).  128 threads with one atom each: three
 // CTAs; their ring evaluation waits for its own chains, and a third CTA hides
 // more of that than 168 registers cost (1,024 x 100 atoms: 4.24 against 4.66
-// ms).  256 threads with two atoms each: two CTAs, 128 registers; the tiled
-// evaluation is bound by latency with eight warps an SM, and sixteen pay for
-// its spills (1,024 x 500 atoms, mixed: 71.2 against 79.7 ms).  512 threads:
-// all registers of one CTA.
+// ms).  512 threads: all registers of one CTA.
+// 256 threads with two atoms each: the tiled evaluation is bound by latency with
+// eight warps an SM, and a second CTA, with 128 registers, pays for its spills
+// (mixed: 1.8 KB of stores; 1,024 x 500 atoms: 60.6 against 75.8 ms) -- where there
+// is one.  Mixed precision has two builds: with no more candidates than SMs one
+// CTA of up to 255 registers, without spills (20 x 300 atoms: 7.5 against 8.7 ms,
+// 152 x 500: 11.1 against 12.9); with more, two (200 x 300: 11.2 against 14.5).  FP64
+// does not spill at 128 registers and is as fast with one CTA as at 214.
 // POT: pair potential (LJ_POT_LJ, Eq. (1); LJ_POT_MORSE).
 constexpr int min_ctas(int T, int A, bool mixed) {
-  return mixed && T <= 64 ? 2 : mixed && T * A <= 128 ? 3 : T * A <= 256 ? 0 : T == 256 ? 2 : 1;
+  return mixed && T <= 64 ? 2 : mixed && T * A <= 128 ? 3 : T * A <= 256 ? 0
+         : !mixed && T == 256 ? 2 : 1;
 }
-template <int T, int A, bool MIXED, int POT = LJ_POT_LJ>
-__global__ void __launch_bounds__(cta_threads_for(T), min_ctas(T, A, MIXED))
+__host__ __device__ constexpr bool two_builds(int T, int A, bool mixed) { return mixed && T == 256 && A == 2; }
+template <int T, int A, bool MIXED, int POT = LJ_POT_LJ, int CTAS = min_ctas(T, A, MIXED)>
+__global__ void __launch_bounds__(cta_threads_for(T), CTAS)
     lbfgs_kernel(ljh::LbfgsArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int TPC = cta_threads_for(T) / T;
+  if constexpr (two_builds(T, A, MIXED))   // a list's candidates go to one of two builds
+    if (a.list_count && (*a.list_count <= a.count_min || *a.list_count > a.count_max)) return;
   const int team = threadIdx.x / T;
   Team<T> tm;
   tm.rank = threadIdx.x % T;
@@ -158,11 +168,14 @@ cudaError_t plan_one(int max_n, int m, int64_t n_cand, int device, ljh::Plan* ou
   const bool on_chip =
       !hist_global && TPC * team_smem_bytes<T>(max_n, buf, hist_bytes) <= kSmemBudget;
   const size_t smem = TPC * team_smem_bytes<T>(max_n, buf, on_chip ? hist_bytes : 0);
-  auto k = lbfgs_kernel<T, A, MIXED, POT>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
-  if (e != cudaSuccess) return e;
   int sms = 0, per_sm = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+  out->many = two_builds(T, A, MIXED) && n_cand > sms ? sms : 0;
+  auto k = lbfgs_kernel<T, A, MIXED, POT>;
+  if constexpr (two_builds(T, A, MIXED))
+    if (out->many) k = lbfgs_kernel<T, A, MIXED, POT, 2>;
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
+  if (e != cudaSuccess) return e;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, smem);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
@@ -234,6 +247,17 @@ cudaError_t plan_impl(int max_n, int m, int64_t n_cand, int device, int team, lj
   });
 }
 
+template <int T, int A, bool MIXED, int POT, int CTAS>
+cudaError_t launch_one(const ljh::LbfgsArgs& a, int grid, size_t smem, cudaStream_t s) {
+  if constexpr (two_builds(T, A, MIXED)) {
+    cudaError_t e = cudaFuncSetAttribute(lbfgs_kernel<T, A, MIXED, POT, CTAS>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
+    if (e != cudaSuccess) return e;
+  }
+  lbfgs_kernel<T, A, MIXED, POT, CTAS><<<grid, cta_threads_for(T), smem, s>>>(a);
+  return cudaGetLastError();
+}
+
 template <bool MIXED, int POT = LJ_POT_LJ>
 cudaError_t launch_impl(const ljh::LbfgsArgs& a, const ljh::Plan& plan, cudaStream_t s) {
   cudaError_t e = cudaMemsetAsync(a.queue, 0, sizeof(unsigned long long), s);
@@ -241,8 +265,20 @@ cudaError_t launch_impl(const ljh::LbfgsArgs& a, const ljh::Plan& plan, cudaStre
   return dispatch_lb(a.max_n, plan.team, [&](auto TT, auto AA) -> cudaError_t {
     constexpr int T = decltype(TT)::value;
     constexpr int A = decltype(AA)::value;
-    lbfgs_kernel<T, A, MIXED, POT><<<plan.grid, cta_threads_for(T), plan.smem, s>>>(a);
-    return cudaGetLastError();
+    if constexpr (two_builds(T, A, MIXED))
+      if (plan.many) {
+        ljh::LbfgsArgs b = a;
+        if (a.list_count) {             // how many there are is known on the device only
+          b.count_max = plan.many;
+          e = launch_one<T, A, MIXED, POT, min_ctas(T, A, MIXED)>(
+              b, std::min(plan.grid, plan.many), plan.smem, s);
+          if (e != cudaSuccess) return e;
+          b.count_max = ~0u;
+          b.count_min = plan.many;
+        }
+        return launch_one<T, A, MIXED, POT, 2>(b, plan.grid, plan.smem, s);
+      }
+    return launch_one<T, A, MIXED, POT, min_ctas(T, A, MIXED)>(a, plan.grid, plan.smem, s);
   });
 }
 
