@@ -608,13 +608,11 @@ __device__ __forceinline__ ff df_sub(ff a, ff b) {
   const ff s = ff_two_sum(a.hi, -b.hi);
   return df_fast_two_sum(s.hi, __fadd_rn(s.lo, __fsub_rn(a.lo, b.lo)));
 }
-// a - b and a b without the last renormalisation, for values that go into
-// df_norm2, a product or df_acc, which take an unnormalised pair: 8 and 4
-// operations instead of 11 and 7
-__device__ __forceinline__ ff df_sub_raw(ff a, ff b) {
-  const ff s = ff_two_sum(a.hi, -b.hi);
-  return ff{s.hi, __fadd_rn(s.lo, __fsub_rn(a.lo, b.lo))};
-}
+// a b without the last renormalisation, for products that are only summed (df_acc):
+// 4 operations instead of 7.  Differences of coordinates are renormalised
+// before they are multiplied: without that, lo is an ulp of the coordinates and
+// not of their difference, and the lo * lo and the roundings that a product drops
+// made pair terms 1.2 (small clusters) to 1.8 times (12 sigma across) less exact.
 __device__ __forceinline__ ff df_mul_raw(ff a, ff b) {
   const ff p = df_two_prod(a.hi, b.hi);
   return ff{p.hi, fmaf(a.lo, b.hi, fmaf(a.hi, b.lo, p.lo))};
@@ -646,11 +644,10 @@ __device__ __forceinline__ ff df_from_double(double x) {
   return ff{h, (float)(x - (double)h)};
 }
 
-// |d|^2 of a double-float vector (not necessarily normalised) with one
-// renormalisation: the high squares exactly (TwoProd by FMA), summed by two
-// TwoSums, and every low-order part (their rounding errors, (2 hi + lo) lo, the
-// TwoProd errors) gathered in one FP32 word, whose roundings are ~2^-47 of the
-// result.
+// |d|^2 of a double-float vector with one renormalisation: the high squares
+// exactly (TwoProd by FMA), summed by two TwoSums, and every low-order part
+// (their rounding errors, (2 hi + lo) lo, the TwoProd errors) gathered in one FP32
+// word, whose roundings are ~2^-47 of the result.
 __device__ __forceinline__ ff df_norm2(ff x, ff y, ff z) {
   const float px = __fmul_rn(x.hi, x.hi), py = __fmul_rn(y.hi, y.hi), pz = __fmul_rn(z.hi, z.hi);
   const float ex = fmaf(x.hi, x.hi, -px), ey = fmaf(y.hi, y.hi, -py), ez = fmaf(z.hi, z.hi, -pz);
@@ -722,9 +719,9 @@ __device__ __forceinline__ ff df_exp(ff x) {
 // (+inf for coincident atoms).  rho is the double-float range parameter.
 __device__ __forceinline__ void pair_term_morse_df(const PosDF& a, const PosDF& b, ff rho,
                                                    ff& vx, ff& vy, ff& vz, ff& e) {
-  const ff dx = df_sub_raw(ff{a.xh, a.xl}, ff{b.xh, b.xl});
-  const ff dy = df_sub_raw(ff{a.yh, a.yl}, ff{b.yh, b.yl});
-  const ff dz = df_sub_raw(ff{a.zh, a.zl}, ff{b.zh, b.zl});
+  const ff dx = df_sub(ff{a.xh, a.xl}, ff{b.xh, b.xl});
+  const ff dy = df_sub(ff{a.yh, a.yl}, ff{b.yh, b.yl});
+  const ff dz = df_sub(ff{a.zh, a.zl}, ff{b.zh, b.zl});
   const ff r2 = df_norm2(dx, dy, dz);
   const ff r = df_sqrt(r2);
   const ff ex = df_exp(df_sub(rho, df_mul(rho, r)));
@@ -965,20 +962,19 @@ __device__ __forceinline__ void pair_term_f64(const PosD& a, const PosD& b, doub
   vx = c * dx; vy = c * dy; vz = c * dz;
 }
 
-// pair term in double-float on coordinates scaled by 1/sigma: with s12 = s6^2,
-// e = s12 - s6 and c = s2 (s12 + e).  v and e are not renormalised (they are
-// summed by df_acc).  123 FP32 operations.
+// pair term in double-float on coordinates scaled by 1/sigma.  v and e are not
+// renormalised (they are summed by df_acc).
 __device__ __forceinline__ void pair_term_df(const PosDF& a, const PosDF& b, ff& vx, ff& vy,
                                              ff& vz, ff& e) {
-  const ff dx = df_sub_raw(ff{a.xh, a.xl}, ff{b.xh, b.xl});
-  const ff dy = df_sub_raw(ff{a.yh, a.yl}, ff{b.yh, b.yl});
-  const ff dz = df_sub_raw(ff{a.zh, a.zl}, ff{b.zh, b.zl});
+  const ff dx = df_sub(ff{a.xh, a.xl}, ff{b.xh, b.xl});
+  const ff dy = df_sub(ff{a.yh, a.yl}, ff{b.yh, b.yl});
+  const ff dz = df_sub(ff{a.zh, a.zl}, ff{b.zh, b.zl});
   const ff r2 = df_norm2(dx, dy, dz);
   const ff s2 = df_rcp(r2);
   const ff s6 = df_mul(df_sqr(s2), s2);
-  const ff s12 = df_sqr(s6);
-  e = df_sub_raw(s12, s6);
-  const ff c = df_mul(s2, df_add(s12, e));
+  const ff t = df_add_f(s6, -1.f);
+  e = df_mul_raw(s6, t);
+  const ff c = df_mul(df_mul(s2, s6), df_add(s6, t));
   vx = df_mul_raw(c, dx); vy = df_mul_raw(c, dy); vz = df_mul_raw(c, dz);
 }
 
