@@ -341,6 +341,7 @@ __global__ void __launch_bounds__(256, POT == LJ_POT_LJ ? 2 : 1) eval_ring_f64_k
 // ---- launch ------------------------------------------------------------------
 constexpr int kRingMaxB = 256;                // largest CTA of both kernels
 constexpr size_t kRingSmem = 104 * 1024;      // shared memory that lets two CTAs share an SM
+constexpr int kUnevenPackedH = 8;             // most shifts of a packed uneven cluster (68 atoms)
 
 struct RingLaunch {
   RingPlan pl;
@@ -356,6 +357,35 @@ constexpr int ring_most_ks(int G, bool parts) {
 }
 static_assert(ring_most_ks(8, false) == 2 && ring_most_ks(4, true) == 5, "shifts per chunk");
 
+// Relative time of a uniform batch of n_cand clusters of n atoms on `sms` SMs:
+// operations of one thread times the warps that a scheduler gets, which is
+// never less than `floor` (a single warp waits for its own chain) and ends in an
+// uneven tail.  An SM gets whole CTAs, so their number is rounded up: 75 large CTAs on
+// 152 SMs take as long as 152 would.  The weights are fitted to 118 shapes (2 to
+// 1,000 atoms, 1 to 65,536 clusters), each in up to 80 layouts: the layout of the
+// least modelled time takes 2% more than the best measured one in the geometric
+// mean, 14% at most.  (A fixed threshold between packed and split batches left up to
+// half of the SMs or 31 of 32 lanes idle beside it: 5,000 x 4 atoms FP64 47 us, now 9;
+// 30,000 x 2 FP32 33, 6; 150 x 300 FP64 734, 365.)
+double ring_time(bool fp32, int n, long long n_cand, int sms, const RingLaunch& r) {
+  const int G = r.G, NG = (n + G - 1) / G, H = NG / 2, parts = r.pl.P * r.pl.S;
+  const bool one = parts == 1;
+  const int k = (H + parts - 1) / parts;               // shifts of a thread
+  double ops;
+  if (fp32) {                                          // packed instructions
+    const double half = one && H > 0 && !(NG & 1) && G == 4 ? 0.5 : 0.0;   // the split shift
+    ops = (k - half) * (9.5 * G * G + 7.0 * G + 12) + (one ? 4.75 * G * G : 0.0) + 36.0 * G + 90;
+    if (r.multi) ops = 1.1 * ops + 300;
+    ops += (r.pl.P > 1 ? 200 : 0) + (r.pl.S > 1 ? 500 + 200 * r.pl.S : 0);
+  } else {                                             // FP64 instructions
+    ops = k * (25.0 * G * G + 20.0 * G) + 50 + (one ? 12.5 * G * (G - 1) : 0.0);
+    ops = ops * (G == 2 ? 1.0 : G == 3 ? 1.05 : 1.2) + (one ? 0 : 100) + (r.pl.S > 1 ? 200 : 0);
+  }
+  const long long ctas = (n_cand + r.pl.C - 1) / r.pl.C * r.pl.S;
+  const double warps = (double)((ctas + sms - 1) / sms) * r.B / 128;   // of a scheduler
+  return ops * (fp32 ? std::max(3.0, warps) + 0.6 : std::max(1.0, warps) + 0.2);
+}
+
 RingLaunch ring_plan(const ljh::EvalArgs& a, int sms) {
   RingLaunch r;
   const int n = a.uniform_n > 0 ? a.uniform_n : a.max_n;
@@ -366,50 +396,51 @@ RingLaunch ring_plan(const ljh::EvalArgs& a, int sms) {
   // the smallest group that fits a CTA; large batches may take a larger one
   r.G = fp32 ? 4 : n <= 2 * kRingMaxB ? 2 : n <= 3 * kRingMaxB ? 3 : 4;
   int NG = (n + r.G - 1) / r.G;
-  // threads that the batch has with one part per candidate, against what
-  // fills the GPU (FP32: 16 warps an SM; FP64: its units are full at 8)
-  const long long want = (long long)sms * (fp32 ? 512 : 256);
-  if (a.uniform_n > 0 && 2 * a.n_cand * NG > want) {
-    // large uniform batch: pack candidates; the group and CTA size with the
-    // least work, idle threads and padding counted (ties: the smaller CTA)
-    double best = 0.0;
-    r.B = 0;
-    auto consider = [&](int G, bool multi) {
-      const int ng = (n + G - 1) / G, h = ng / 2;
-      if (fp32 && !multi && h > ring_most_ks(G, false)) return;
-      // operations of a thread: pairs, the reaction's sums, energies, and what
-      // it does once for its group (FP32: in packed instructions)
-      const bool half = !(ng & 1) && G <= 4;              // a split shift costs half
-      const double shifts = h - (half && h > 0 ? 0.5 : 0.0);
-      const double ops = fp32 ? shifts * (9.5 * G * G + 7.0 * G + 12) + 4.75 * G * G + 36.0 * G + 90
-                              : shifts * (22.5 * G * G + 6.0 * G) + 11.0 * G * (G - 1) + 20;
-      for (int B = fp32 ? 64 : 96; B <= (fp32 ? 256 : 192) || r.B == 0; B += 32) {
-        const int used = B / ng * ng;
-        if (used == 0) continue;
-        const double cost = ops * ng * B / used;
-        if (r.B == 0 || cost < 0.985 * best) {
-          best = cost; r.B = B; r.G = G; r.multi = multi;
-        }
+  if (a.uniform_n > 0) {
+    RingLaunch best = r;
+    double least = 0.0;
+    auto consider = [&](int G, int C, int P, int S, int B, bool multi) {
+      RingLaunch o = r;
+      o.G = G;
+      o.B = B;
+      o.multi = multi;
+      o.pl.C = C;
+      o.pl.P = P;
+      o.pl.S = S;
+      const double t = ring_time(fp32, n, a.n_cand, sms, o);
+      if (least == 0.0 || t < least || (t == least && B < best.B)) {
+        least = t;
+        best = o;
       }
     };
-    if (fp32) {
-      consider(4, false);
-      consider(8, false);
-      if (r.B == 0) consider(4, true);
-    } else {
-      for (int G = r.G; G <= 4; ++G) consider(G, true);
+    // one part, several candidates a CTA (FP32: of 64 threads; larger ones were never
+    // more than 1% faster, and up to 9% slower where they leave fewer threads idle)
+    for (int G = r.G; G <= (fp32 ? 8 : 4); G += fp32 ? 4 : 1) {
+      const int ng = (n + G - 1) / G;
+      if (fp32 && ng / 2 > ring_most_ks(G, false)) continue;
+      for (int B = fp32 ? 64 : 32; B <= (fp32 ? 64 : 128); B += 32)
+        if (B >= ng) consider(G, B / ng, 1, 1, B, !fp32);
     }
+    // a candidate in parts, over one CTA or several
+    for (int G = r.G; G <= 4; G += std::max(1, 4 - G)) {
+      const int ng = (n + G - 1) / G, h = ng / 2;
+      for (int P : {1, 2, 3, 4, 5, 6, 8, 10}) {
+        if ((P > 1 && P > h + 1) || ng * P > kRingMaxB) break;
+        for (int fill : {64, 128}) {
+          const int C = fp32 ? std::max(1, fill / (ng * P)) : 1;
+          const int B = (ng * P * C + 31) / 32 * 32;
+          for (int S = 1; S <= 8 && (S == 1 || (C == 1 && h >= S * P)); S *= 2)
+            consider(G, C, P, S, B, true);
+          if (C == 1) break;
+        }
+      }
+    }
+    r = best;
     NG = (n + r.G - 1) / r.G;
-    pl.C = r.B / NG;
-  } else if (a.uniform_n > 0) {
-    // few candidates: more parts until the threads fill the GPU
-    const long long more = want / (a.n_cand * NG);
-    pl.P = (int)std::max(1LL, std::min<long long>(std::min(more, (long long)NG / 2 + 1), kRingMaxB / NG));
-    r.B = (NG * pl.P + 31) / 32 * 32;
-  } else if (fp32 && NG / 2 <= ring_most_ks(4, false) && 2 * a.n_cand * NG > want) {
+  } else if (fp32 && NG / 2 <= kUnevenPackedH && a.n_cand * NG > 64LL * sms) {
     // large uneven batch of small clusters: packed like a uniform one, every
     // candidate with the threads of the largest (33,563 of 4..9 atoms: 22 us a
-    // call, 55 with a CTA each)
+    // call, 55 with a CTA each; 20,000 of 15..60: 35, 70)
     r.B = 64;
     pl.C = r.B / NG;
     r.multi = false;
@@ -422,16 +453,16 @@ RingLaunch ring_plan(const ljh::EvalArgs& a, int sms) {
     pl.P = 2;                                // (reserves the parts' buffer)
   }
   const int H = NG / 2;
-  // CTAs per candidate, while there are fewer than four per SM to share out
-  // and each keeps eight shifts a part
-  if (r.multi && pl.C == 1) {
-    const int P = a.uniform_n > 0 ? pl.P : r.B / NG;
-    while (pl.S < 8 && a.n_cand * pl.S < 4LL * sms && H >= 16 * pl.S * P) pl.S *= 2;
-  }
+  // uneven, few candidates: several CTAs each, while there are fewer than four per SM to
+  // share out and each keeps eight shifts a part
+  if (a.uniform_n <= 0 && r.multi)
+    while (pl.S < 8 && a.n_cand * pl.S < 4LL * sms && H >= 16 * pl.S * (r.B / NG)) pl.S *= 2;
   // shifts between barriers, in equal chunks: FP32 as many as leave shared
-  // memory for 16 warps an SM, FP64 up to five for two CTAs an SM
+  // memory for 16 warps an SM, FP64 up to five for two CTAs an SM; packed ones
+  // take all at once
   const int per = pl.P * pl.S, all = std::max(1, (H + per - 1) / per);
-  for (int most = fp32 ? ring_most_ks(r.G, per > 1) : 5; most >= 1; --most) {
+  pl.KS = all;
+  for (int most = fp32 ? ring_most_ks(r.G, per > 1) : 5; r.multi && most >= 1; --most) {
     const int chunks = (all + most - 1) / most;
     pl.KS = (all + chunks - 1) / chunks;
     if (fp32 || ring_smem(r.B, pl, false, r.G) <= kRingSmem) break;
