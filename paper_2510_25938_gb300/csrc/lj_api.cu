@@ -420,7 +420,7 @@ lj_status lbfgs_minimize_batched(lj_ctx* ctx, const lj_batch* batch, const lj_lb
     const int team = ctx->lbfgs_team ? ctx->lbfgs_team : ctx->tune_team[bucket_of(bound)];
     const bool hg = hist_global_for(ctx, bucket_of(bound));
     return ljh::lbfgs_plan(mixed, p->potential, bound, p->m, batch->n_cand, ctx->device, team,
-                           pl, hg);
+                           pl, hg ? ljh::HIST_GLOBAL : ljh::HIST_AUTO);
   };
   if (batch->uniform_n == 0 && max_n > 32 && batch->n_cand > 1) {
     // Uneven batch spanning several size classes: sort candidates into size
@@ -703,7 +703,7 @@ struct Tuner {
     *df = 0;
     ljh::Plan pl;
     cudaError_t e = ljh::lbfgs_plan(prec == LJ_PREC_MIXED, LJ_POT_LJ, nt, m, nc, ctx->device,
-                                    *team, &pl, false);
+                                    *team, &pl);
     if (e != cudaSuccess) return fail(ctx, LJ_ERR_CUDA, "autotune: plan failed");
     if (pl.hist_on_chip) {                 // the alternative: history in global memory
       ctx->hist_opt = 1;
@@ -996,7 +996,7 @@ lj_status lbfgs_minimize_batched_noalloc(const lj_batch* batch, const lj_lbfgs_p
   ljh::Plan plans[ljh::kMaxBuckets];
   for (int b = 0; b < nb; ++b) {
     cudaError_t e = ljh::lbfgs_plan(mixed, p->potential, bk.bound[b], p->m, batch->n_cand, dev, 0,
-                                    &plans[b]);
+                                    &plans[b], ljh::HIST_CHIP);
     if (e != cudaSuccess) return LJ_ERR_CUDA;
     if (!plans[b].hist_on_chip) {
       // launch only as many teams as the scratch holds history slots for

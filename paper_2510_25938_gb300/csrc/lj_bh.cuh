@@ -83,8 +83,8 @@ __global__ void __launch_bounds__(T, T <= 64 ? 3 : 0) bh_cluster_kernel(ljh::BhA
   void* hbuf;
   void* hist;
   long long* word;
-  carve_team<T>(sp, n, pair_buffer(n, MIXED), a.hist_on_chip ? a.hist_slot_bytes : 0, pos,
-                hbuf, hist, tm.red, word);
+  carve_team<T>(sp, n, pair_buffer(n, MIXED), a.hist_on_chip ? a.hist_slot_bytes : 0,
+                ring_shifts(n), pos, hbuf, hist, tm.red, word);
   MinParams p = to_dev(a.p);
   // hbuf: pairs up to 64 atoms, ring chunks up to 256 (mixed)
   p.layout = pair_layout(n);
@@ -241,12 +241,14 @@ cudaError_t plan_one(int n_atoms, int m, int n_walkers, int K, ljh::Plan* out, b
   if (K <= LJ_MAX_K) {                // one cluster of K CTAs per walker
     const bool buf = pair_buffer(n_atoms, MIXED);
     const bool on_chip = !hist_global && bhc_head_bytes<T>(n_atoms) +
-                                             team_smem_bytes<T>(n_atoms, buf, out->slot_bytes) <=
+                                             team_smem_bytes<T>(n_atoms, buf, out->slot_bytes,
+                                                                ring_shifts(n_atoms)) <=
                                          kSmemBudget;
     out->hist_on_chip = on_chip ? 1 : 0;
     out->slots = on_chip ? 0 : (int64_t)n_walkers * K;
     const size_t smem = bhc_head_bytes<T>(n_atoms) +
-                        team_smem_bytes<T>(n_atoms, buf, on_chip ? out->slot_bytes : 0);
+                        team_smem_bytes<T>(n_atoms, buf, on_chip ? out->slot_bytes : 0,
+                                           ring_shifts(n_atoms));
     auto k = bh_cluster_kernel<T, A, MIXED, POT>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
     if (e != cudaSuccess) return e;

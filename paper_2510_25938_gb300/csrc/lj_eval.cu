@@ -379,7 +379,7 @@ double ring_time(bool fp32, int n, long long n_cand, int sms, const RingLaunch& 
     ops += (r.pl.P > 1 ? 200 : 0) + (r.pl.S > 1 ? 500 + 200 * r.pl.S : 0);
   } else {                                             // FP64 instructions
     ops = k * (25.0 * G * G + 20.0 * G) + 50 + (one ? 12.5 * G * (G - 1) : 0.0);
-    ops = ops * (G == 2 ? 1.0 : G == 3 ? 1.05 : 1.2) + (one ? 0 : 100) + (r.pl.S > 1 ? 200 : 0);
+    ops = ops * (G == 2 ? 1.0 : G == 3 ? 1.15 : 1.25) + (one ? 0 : 100) + (r.pl.S > 1 ? 200 : 0);
   }
   const long long ctas = (n_cand + r.pl.C - 1) / r.pl.C * r.pl.S;
   const double warps = (double)((ctas + sms - 1) / sms) * r.B / 128;   // of a scheduler

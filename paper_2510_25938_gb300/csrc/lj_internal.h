@@ -97,18 +97,23 @@ struct Plan {
                           // candidates is meant (0: the other, or there is only one)
 };
 
+// Where the L-BFGS history goes (results do not depend on it).  HIST_AUTO: on
+// chip within kSmemBudget.  HIST_CHIP: on chip as long as two CTAs fit on an SM; for
+// callers whose global scratch holds fewer histories than teams could run.
+enum HistPlace : int { HIST_AUTO, HIST_GLOBAL, HIST_CHIP };
+
 // largest atom count this build supports
 constexpr int kMaxAtoms = LJ_MAX_ATOMS;
 
 cudaError_t eval_launch(const EvalArgs& a, cudaStream_t s);
 // team: threads per candidate requested for clusters of up to 64 atoms
 // (32, 64 or 128); any other value picks the default for the cluster size.
-// hist_global: keep the L-BFGS history in global memory even where it would
+// hist_global (HIST_GLOBAL): keep the L-BFGS history in global memory even where it would
 // fit in shared memory (a tuning choice; results do not change)
 cudaError_t lbfgs_plan_fp64(int max_n, int m, int64_t n_cand, int device, int team, Plan* out,
-                            bool hist_global = false);
+                            HistPlace hist = HIST_AUTO);
 cudaError_t lbfgs_plan_mixed(int max_n, int m, int64_t n_cand, int device, int team, Plan* out,
-                             bool hist_global = false);
+                             HistPlace hist = HIST_AUTO);
 cudaError_t lbfgs_launch_fp64(const LbfgsArgs& a, const Plan& plan, cudaStream_t s);
 cudaError_t lbfgs_launch_mixed(const LbfgsArgs& a, const Plan& plan, cudaStream_t s);
 // sort candidates of an uneven batch into size buckets (device, no sync)
@@ -126,9 +131,9 @@ cudaError_t bh_launch_mixed(const BhArgs& a, const Plan& plan, cudaStream_t s);
 
 // the same kernels on the Morse pair potential (lj_morse_*.cu)
 cudaError_t lbfgs_plan_morse_fp64(int max_n, int m, int64_t n_cand, int device, int team,
-                                  Plan* out, bool hist_global);
+                                  Plan* out, HistPlace hist);
 cudaError_t lbfgs_plan_morse_mixed(int max_n, int m, int64_t n_cand, int device, int team,
-                                   Plan* out, bool hist_global);
+                                   Plan* out, HistPlace hist);
 cudaError_t lbfgs_launch_morse_fp64(const LbfgsArgs& a, const Plan& plan, cudaStream_t s);
 cudaError_t lbfgs_launch_morse_mixed(const LbfgsArgs& a, const Plan& plan, cudaStream_t s);
 cudaError_t bh_plan_morse_fp64(int n_atoms, int m, int n_walkers, int K, int team, Plan* out,
@@ -140,12 +145,12 @@ cudaError_t bh_launch_morse_mixed(const BhArgs& a, const Plan& plan, cudaStream_
 
 // plan / launch by precision and pair potential
 inline cudaError_t lbfgs_plan(bool mixed, int pot, int max_n, int m, int64_t n_cand, int device,
-                              int team, Plan* out, bool hist_global = false) {
+                              int team, Plan* out, HistPlace hist = HIST_AUTO) {
   if (pot == LJ_POT_MORSE)
-    return mixed ? lbfgs_plan_morse_mixed(max_n, m, n_cand, device, team, out, hist_global)
-                 : lbfgs_plan_morse_fp64(max_n, m, n_cand, device, team, out, hist_global);
-  return mixed ? lbfgs_plan_mixed(max_n, m, n_cand, device, team, out, hist_global)
-               : lbfgs_plan_fp64(max_n, m, n_cand, device, team, out, hist_global);
+    return mixed ? lbfgs_plan_morse_mixed(max_n, m, n_cand, device, team, out, hist)
+                 : lbfgs_plan_morse_fp64(max_n, m, n_cand, device, team, out, hist);
+  return mixed ? lbfgs_plan_mixed(max_n, m, n_cand, device, team, out, hist)
+               : lbfgs_plan_fp64(max_n, m, n_cand, device, team, out, hist);
 }
 inline cudaError_t lbfgs_launch(const LbfgsArgs& a, const Plan& plan, cudaStream_t s) {
   if (a.p.k.pot == LJ_POT_MORSE)

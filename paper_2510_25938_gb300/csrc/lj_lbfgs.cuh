@@ -63,15 +63,16 @@ __global__ void __launch_bounds__(cta_threads_for(T), CTAS)
   void* hist;
   const size_t hb = a.hist_on_chip ? a.hist_slot_bytes : 0;
   const bool buf = pair_buffer(a.max_n, MIXED);
-  carve_team<T>(smem + team * team_smem_bytes<T>(a.max_n, buf, hb), a.max_n, buf, hb, pos, hbuf,
-                hist, tm.red, word);
+  const int ks = ring_shifts(a.max_n, a.p.m);
+  carve_team<T>(smem + team * team_smem_bytes<T>(a.max_n, buf, hb, ks), a.max_n, buf, hb, ks, pos,
+                hbuf, hist, tm.red, word);
   MinParams p = to_dev(a.p);
   // hbuf: pairs up to 64 atoms, ring chunks up to 256 (mixed), tile accumulators above.  With
   // one-sided rows chosen above 256 atoms there is no pair buffer to use: the
   // buffer holds 24 bytes per atom, not per pair, so it is withdrawn and every
   // tier evaluates in one-sided rows
   p.layout = pair_layout(a.max_n);
-  p.ring_ks = ring_shifts(a.max_n);
+  p.ring_ks = ks;
   if (a.max_n > kTileMinN && a.p.df_one_sided) hbuf = nullptr;
   const long long slot = (long long)blockIdx.x * TPC + team;
   if (!a.hist_on_chip) hist = static_cast<unsigned char*>(a.hist) + slot * a.hist_slot_bytes;
@@ -160,14 +161,16 @@ __global__ void __launch_bounds__(cta_threads_for(T), CTAS)
 
 template <int T, int A, bool MIXED, int POT>
 cudaError_t plan_one(int max_n, int m, int64_t n_cand, int device, ljh::Plan* out,
-                     bool hist_global) {
+                     ljh::HistPlace place) {
   constexpr int threads = cta_threads_for(T);
   constexpr int TPC = threads / T;
   const size_t hist_bytes = align16(2 * (size_t)m * A * 3 * T * (MIXED ? sizeof(float) : sizeof(double)));
   const bool buf = pair_buffer(max_n, MIXED);
+  const int ks = ring_shifts(max_n, m);
   const bool on_chip =
-      !hist_global && TPC * team_smem_bytes<T>(max_n, buf, hist_bytes) <= kSmemBudget;
-  const size_t smem = TPC * team_smem_bytes<T>(max_n, buf, on_chip ? hist_bytes : 0);
+      place != ljh::HIST_GLOBAL && TPC * team_smem_bytes<T>(max_n, buf, hist_bytes, ks) <=
+                                       (place == ljh::HIST_CHIP ? kSmemTwo : kSmemBudget);
+  const size_t smem = TPC * team_smem_bytes<T>(max_n, buf, on_chip ? hist_bytes : 0, ks);
   int sms = 0, per_sm = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
   out->many = two_builds(T, A, MIXED) && n_cand > sms ? sms : 0;
@@ -240,10 +243,10 @@ cudaError_t dispatch_lb(int max_n, int team, F&& f) {
 
 template <bool MIXED, int POT = LJ_POT_LJ>
 cudaError_t plan_impl(int max_n, int m, int64_t n_cand, int device, int team, ljh::Plan* out,
-                      bool hist_global) {
+                      ljh::HistPlace place) {
   return dispatch_lb(max_n, team, [&](auto TT, auto AA) -> cudaError_t {
     return plan_one<decltype(TT)::value, decltype(AA)::value, MIXED, POT>(max_n, m, n_cand, device,
-                                                                          out, hist_global);
+                                                                          out, place);
   });
 }
 

@@ -48,8 +48,8 @@ cudaError_t tune_starts_launch(double* x, int64_t n_cand, int n, double side, ui
 }
 
 cudaError_t lbfgs_plan_fp64(int max_n, int m, int64_t n_cand, int device, int team, Plan* out,
-                            bool hist_global) {
-  return ljlb::plan_impl<false>(max_n, m, n_cand, device, team, out, hist_global);
+                            HistPlace hist) {
+  return ljlb::plan_impl<false>(max_n, m, n_cand, device, team, out, hist);
 }
 
 cudaError_t lbfgs_launch_fp64(const LbfgsArgs& a, const Plan& plan, cudaStream_t s) {

@@ -5,8 +5,8 @@
 namespace ljh {
 
 cudaError_t lbfgs_plan_morse_fp64(int max_n, int m, int64_t n_cand, int device, int team,
-                                  Plan* out, bool hist_global) {
-  return ljlb::plan_impl<false, LJ_POT_MORSE>(max_n, m, n_cand, device, team, out, hist_global);
+                                  Plan* out, HistPlace hist) {
+  return ljlb::plan_impl<false, LJ_POT_MORSE>(max_n, m, n_cand, device, team, out, hist);
 }
 
 cudaError_t lbfgs_launch_morse_fp64(const LbfgsArgs& a, const Plan& plan, cudaStream_t s) {

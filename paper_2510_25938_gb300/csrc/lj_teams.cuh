@@ -47,14 +47,26 @@ __host__ __device__ constexpr int pair_layout(int max_n) {
 __host__ __device__ constexpr bool pair_buffer(int max_n, bool mixed) {
   return mixed || pair_layout(max_n) != LAYOUT_RING;
 }
-// shifts of a ring chunk: the history of up to 256 atoms (m = 10, FP32) stays
-// on chip beside it
-__host__ __device__ constexpr int ring_shifts(int max_n) { return max_n <= 128 ? 8 : 4; }
+// Shared memory of a CTA that leaves room for a second one on the SM.
+constexpr size_t kSmemTwo = 113 * 1024;
 
-__host__ __device__ constexpr size_t half_bytes(int max_n, bool half) {
+// Shifts of a ring chunk: the history of up to 256 atoms (m = 10, FP32) stays on
+// chip beside it.  L-BFGS with a longer one (m > 27 up to 128 atoms, m > 13 above): as
+// many shifts, but two at least, as leave it within kSmemTwo, where HIST_CHIP keeps it
+// (1,024 x 128 atoms, m = 31, without allocation: 6.7 ms, 9.4 with the history in the
+// fixed scratch, 8.1 before the ring).  The number belongs to the sizes and not
+// to the place, since the order of the sums follows it.
+__host__ __device__ constexpr int ring_shifts(int max_n, int m = 0) {
+  const int most = max_n <= 128 ? 8 : 4, slots = max_n <= 128 ? 128 : 256;
+  const long long left = (long long)kSmemTwo - 1024 - 32LL * max_n - 24LL * m * slots;
+  const long long fit = left / (24LL * max_n);
+  return fit >= most || fit < 2 ? most : (int)fit;
+}
+
+__host__ __device__ constexpr size_t half_bytes(int max_n, bool half, int ks) {
   return !half ? 0
          : align16((size_t)24 * (pair_layout(max_n) == LAYOUT_HALF   ? max_n * (max_n - 1) / 2
-                                 : pair_layout(max_n) == LAYOUT_RING ? max_n * ring_shifts(max_n)
+                                 : pair_layout(max_n) == LAYOUT_RING ? max_n * ks
                                                                      : max_n));
 }
 
@@ -63,18 +75,19 @@ __host__ __device__ constexpr size_t half_bytes(int max_n, bool half) {
 // L-BFGS history (hist_bytes > 0: kept on chip instead of in the workspace),
 // cross-warp reduction scratch (double-buffered), one word
 template <int T>
-__host__ __device__ constexpr size_t team_smem_bytes(int max_n, bool half, size_t hist_bytes = 0) {
-  return align16((size_t)max_n * sizeof(PosD)) + half_bytes(max_n, half) + align16(hist_bytes) +
+__host__ __device__ constexpr size_t team_smem_bytes(int max_n, bool half, size_t hist_bytes,
+                                                             int ks) {
+  return align16((size_t)max_n * sizeof(PosD)) + half_bytes(max_n, half, ks) + align16(hist_bytes) +
          (T > 32 ? 2 * 8 * (T / 32) * sizeof(double) : 0) + 16;
 }
 
 template <int T>
 __device__ __forceinline__ void carve_team(unsigned char* base, int max_n, bool half,
-                                           size_t hist_bytes, void*& pos, void*& hbuf,
+                                           size_t hist_bytes, int ks, void*& pos, void*& hbuf,
                                            void*& hist, double*& red, long long*& word) {
   pos = base;
   unsigned char* p = base + align16((size_t)max_n * sizeof(PosD));
-  const size_t hb = half_bytes(max_n, half);
+  const size_t hb = half_bytes(max_n, half, ks);
   hbuf = hb ? static_cast<void*>(p) : nullptr;
   p += hb;
   hist = hist_bytes ? static_cast<void*>(p) : nullptr;
