@@ -255,6 +255,10 @@ const char* lj_ctx_last_error(const lj_ctx* ctx);
  *   d_energy [n_cand] FP64 energies.
  *   d_grad [total_atoms*3] gradient dE/dx in xtype, or NULL for energy only.
  *   eps, sigma  Eq. (1) parameters (> 0).
+ * Deterministic: the same call gives the same bits.  The order of the sums
+ * follows the batch (its number of candidates and their largest size decide how
+ * a candidate is spread over threads), so the same cluster alone, in a shard
+ * or in another batch can differ in its last bits.
  */
 lj_status lj_energy_grad_batched(lj_ctx* ctx, const lj_batch* batch, lj_precision prec,
                                  lj_dtype xtype, const void* d_x, double* d_energy,

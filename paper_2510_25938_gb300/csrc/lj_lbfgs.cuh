@@ -29,7 +29,7 @@ __device__ __forceinline__ MinParams to_dev(const ljh::MinParamsH& h) {
 // Register budget.  Mixed precision, teams of up to 64 threads: two CTAs of 128
 // threads an SM, 255 registers; left to itself the compiler stops at 168 with
 // spills, and the third CTA that this leaves room for does not make up for them
-// (4,096 x LJ38: 2.64 against 2.82 ms).  128 threads with one atom each: three
+// (4,096 x LJ38, earlier forms of the evaluation: 2.64 against 2.82 ms).  128 threads with one atom each: three
 // CTAs; their ring evaluation waits for its own chains, and a third CTA hides
 // more of that than 168 registers cost (1,024 x 100 atoms: 4.24 against 4.66
 // ms).  512 threads: all registers of one CTA.

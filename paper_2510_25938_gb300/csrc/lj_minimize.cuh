@@ -121,8 +121,12 @@ __device__ __forceinline__ int hidx(int slot, int a, int c, int rank) {
 // ---------------------------------------------------------------------------
 // PM = 0: pair terms in X precision; PM = 1 (X = double only): pair terms in
 // double-float arithmetic on coordinates scaled by 1/sigma.
-// hbuf: the team's half-pair buffer (24 bytes per pair) or nullptr; used for
-// FP64 / double-float evaluations, which then compute each pair once.
+// hbuf: the team's pair buffer, laid out as p.layout says, or nullptr (FP64 path from
+// 65 to 256 atoms, one-sided rows chosen above); FP64 and double-float
+// evaluations with one compute each pair once, others in one-sided rows.
+// Mixed-precision teams of up to 256 atoms always have one; their rows stay compiled
+// because without them the rest is scheduled worse (LJ38 Basin Hopping, 64 walkers x
+// 8, 25 steps: 10.48 against 10.14 ms).
 // ---------------------------------------------------------------------------
 // Morse pair potential (Morse 1929, cluster form), the pair-potential
 // extension of the method: V(r) = eps e (e - 2), e = exp(rho (1 - r / re)),
@@ -132,7 +136,8 @@ __device__ __forceinline__ int hidx(int slot, int a, int c, int rank) {
 // g_i = -(2 eps rho / re) sum_{j != i} e (e - 1) (x_i - x_j) / r.
 // FP32 (first tier of the mixed path; compensated energy), double-float
 // (evaluate_morse_df, the polish tier) and FP64; those two take each pair once
-// through the team's buffer up to 256 atoms, as for Eq. (1) (half pairs, ring).
+// through the team's buffer where there is one, up to 256 atoms, as for Eq. (1)
+// (half pairs, ring).
 // Coincident atoms give E = +inf (and a non-finite gradient), as for Eq. (1).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ float to_value(ff v) { return v.hi + v.lo; }
@@ -784,7 +789,7 @@ __device__ __forceinline__ void warp_sum2(V& v0, V& v1) {
 // block of two pairs, 175 of them the two-value reduction, and ~570 once.
 // LJ38 Basin Hopping near its minima (64 walkers x 8, 25 steps, mixed): 11.8 ms a
 // launch before this form, one evaluation in the line search (run_phase) and the
-// ring order of the half pairs, 9.9 after.
+// ring order of the half pairs, 10.1 after.
 // ---------------------------------------------------------------------------
 // a lane's part of a vector, of a dot product and of an update: FP32 16 bytes,
 // two values an instruction; FP64 one value
@@ -1406,7 +1411,7 @@ __device__ __forceinline__ int run_phase(const Team<T>& tm, int n, typename P::X
 // Minimise the cluster whose owned coordinates are in x64 (in place).
 // hist: this team's history slot (2 m A 3 T values of the phase's V type).
 // pos:  this team's shared position buffer (n entries of 32 bytes).
-// hbuf: this team's half-pair buffer (24 n(n-1)/2 bytes) or nullptr.
+// hbuf: this team's pair buffer (see evaluate) or nullptr.
 // MIXED: FP32 phase, then polish iterations whose evaluations run in
 // double-float arithmetic; convergence is confirmed, and the returned energy
 // computed, by a true FP64 evaluation (if FP64 disagrees, polishing goes on).

@@ -36,7 +36,7 @@ using namespace ljd;
 namespace cg = cooperative_groups;
 
 struct RingPlan {
-  int C;       // candidates per CTA (uniform batches; uneven: 1)
+  int C;       // candidates per CTA (uniform and packed uneven batches; other uneven ones: 1)
   int P;       // parts of a candidate in a CTA (uneven: as many as fit, per candidate)
   int S;       // CTAs per candidate (cluster size)
   int KS;      // shifts between two barriers
@@ -118,7 +118,6 @@ __device__ __forceinline__ ff e2_total(const E2& e) {
   return ff{t.hi, __fadd_rn(t.lo, __fadd_rn(e.lo.x, e.lo.y))};
 }
 __device__ __forceinline__ V2 v2_zero() { return V2{f2(0.f), f2(0.f), f2(0.f)}; }
-__device__ __forceinline__ V2 v2_dup(float x, float y, float z) { return V2{f2(x), f2(y), f2(z)}; }
 __device__ __forceinline__ void v2_add(V2& a, const V2& b) {
   a.x = __fadd2_rn(a.x, b.x); a.y = __fadd2_rn(a.y, b.y); a.z = __fadd2_rn(a.z, b.z);
 }
