@@ -81,7 +81,7 @@ FP64_PEAK_TFLOPS = 1.25                    # nominal FP64 (non-tensor) rate of G
 # dram__bytes_read.sum + dram__bytes_write.sum of one bh_cluster_kernel launch of this
 # workload (25 BH steps), from one ncu capture of the launch as the bench makes it; None
 # whenever the kernel or the launch changes until it is captured again
-BH_DRAM_BYTES_PER_LAUNCH = None
+BH_DRAM_BYTES_PER_LAUNCH = 958464
 
 
 def parse():
